@@ -192,6 +192,7 @@ mg_status alloc_workspaces(Handle& H, cudaStream_t s, bool owner) {
     MG_TRY(halloc_t(H, &H.uvec, KLD));
     MG_TRY(halloc_t(H, &H.dr, 1));
     if (owner) MG_TRY(halloc_t(H, &H.pls, 1));
+    if (owner) MG_TRY(halloc_t(H, &H.pmat, 1));
     H.cpart_ctas = sm_count();
     MG_TRY(halloc_t(H, &H.cpart, (size_t)2 * H.cpart_ctas * PSTR));
     MG_TRY(halloc_t(H, &H.cstats, 1));
@@ -215,6 +216,7 @@ mg_status alloc_workspaces(Handle& H, cudaStream_t s, bool owner) {
         if (owner) {
             MG_TRY(halloc_t(H, &H.fdW, (size_t)(p.dr_m + 1) * n0));
             MG_TRY(halloc_t(H, &H.fdpls, 1));
+            MG_TRY(halloc_t(H, &H.fdpmat, 1));
         }
     }
     return MG_OK;
@@ -349,9 +351,11 @@ mg_status make_context(Handle& P, mg_handle_s** out) {
     C.c64.W = P.c64.W;
     C.c32.W = P.c32.W;
     C.pls = P.pls;
+    C.pmat = P.pmat;
     C.defl_k = P.defl_k;
     C.fdW = P.fdW;
     C.fdpls = P.fdpls;
+    C.fdpmat = P.fdpmat;
     C.fine_k = P.fine_k;
     auto fail = [&](mg_status st) {
         for (void* q : C.allocs) cudaFree(q);

@@ -36,7 +36,7 @@ CoopArgs<T> coarse_args(Handle& H, const C2<T>* f, C2<T>* x, C2<T>* r, C2<T>* V,
     a.r = r;
     a.V = V;
     a.W = H.coarse<T>().W;
-    a.pls = H.pls;
+    a.pm = H.pmat;
     a.k = H.defl_k;
     a.ms = std::max(H.p.dr_m - H.defl_k, 1);
     a.tol = tol;
@@ -72,6 +72,7 @@ mg_status mg_set_deflation(mg_handle h, const void* W, const void* Hm, int k) {
     double2* hk = MG_DEVF(H.dr, double2, Hk);
     MG_CUDA_TRY(cudaMemcpy(hk, colmaj.data(), colmaj.size() * sizeof(double2), cudaMemcpyHostToDevice));
     ks_load_dense(H.pls, hk, nullptr, k, 0.0, s);
+    proj_mats(H.pls, H.pmat, k, s);
     launch_convert<double, float>(H.c32.W, H.c64.W, (long)(k + 1) * n2, Gate{}, s);
     MG_LAUNCH_CHECK();
     MG_CUDA_TRY(cudaStreamSynchronize(s));

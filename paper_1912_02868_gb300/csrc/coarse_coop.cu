@@ -701,33 +701,13 @@ __global__ void __maxnreg__(128) k_coarse_proj(CoopArgs<T> a) {
         }
 
     // Projection onto the deflation space, d = argmin ||W^+ r - H_k d||, as two
-    // small matrices fixed for the whole solve: d = M g and H_k d = N g with
-    // g = W^+ r, M = R^{-1} Q^+ from the QR factorisation of H_k (the stored
-    // rotations and R), N = H_k M.  Warp 0 builds column l of both by solving
-    // for g = e_l.
+    // small matrices: d = M g and H_k d = N g with g = W^+ r (ProjMats), copied once
+    // into shared memory.
     Z* Mp = reinterpret_cast<Z*>(smem_raw + sizeof(ClusterSmem<T>) +
                                  (a.vs ? slice_bytes<T>(ms, a.spc * NDOF) : 0));
     Z* Np = Mp + k * (k + 1);
-    if (tid < 32) {
-        const KState* P = a.pls;
-        for (int l = tid; l <= k; l += 32) {
-            Z g[KLD], dd[KMAX];
-            for (int i = 0; i <= k; ++i) g[i] = mk<T>(i == l ? T(1) : T(0), 0);
-            for (int t = 0; t < P->nrot; ++t)
-                rot_<T>((T)P->rc[t], from_d2<T>(P->rs[t]), g[P->ra[t]], g[P->rb[t]]);
-            for (int i = k - 1; i >= 0; --i) {
-                Z acc = g[i];
-                for (int m = i + 1; m < k; ++m) acc = cfms_<T>(from_d2<T>(P->R[i + KLD * m]), dd[m], acc);
-                dd[i] = cdiv_<T>(acc, from_d2<T>(P->R[i + KLD * i]));
-            }
-            for (int i = 0; i < k; ++i) Mp[i + k * l] = dd[i];
-            for (int i = 0; i <= k; ++i) {
-                Z acc = mk<T>(0, 0);
-                for (int m = 0; m < k; ++m) acc = cfma(from_d2<T>(P->H[i + KLD * m]), dd[m], acc);
-                Np[i + (k + 1) * l] = acc;
-            }
-        }
-    }
+    for (int e = tid; e < k * (k + 1); e += nt) Mp[e] = from_d2<T>(a.pm->M[e]);
+    for (int e = tid; e < (k + 1) * (k + 1); e += nt) Np[e] = from_d2<T>(a.pm->N[e]);
 
     // a.ash: the FP16 blocks of the first ASH_DIRS directions of the own sites,
     // copied once into shared memory after M and N
@@ -1447,26 +1427,8 @@ __global__ void __maxnreg__(128) k_coarse_proj_pair(CoopArgs<T> a0, CoopArgs<T> 
     // projection matrices M, N (shared deflation space), as in k_coarse_proj
     Z* Mp = Vb[1] + (long)(ms + 1) * rows_cap;
     Z* Np = Mp + k * (k + 1);
-    if (tid < 32) {
-        const KState* P = a0.pls;
-        for (int l = tid; l <= k; l += 32) {
-            Z g[KLD], dd[KMAX];
-            for (int i = 0; i <= k; ++i) g[i] = mk<T>(i == l ? T(1) : T(0), 0);
-            for (int t = 0; t < P->nrot; ++t)
-                rot_<T>((T)P->rc[t], from_d2<T>(P->rs[t]), g[P->ra[t]], g[P->rb[t]]);
-            for (int i = k - 1; i >= 0; --i) {
-                Z acc = g[i];
-                for (int m = i + 1; m < k; ++m) acc = cfms_<T>(from_d2<T>(P->R[i + KLD * m]), dd[m], acc);
-                dd[i] = cdiv_<T>(acc, from_d2<T>(P->R[i + KLD * i]));
-            }
-            for (int i = 0; i < k; ++i) Mp[i + k * l] = dd[i];
-            for (int i = 0; i <= k; ++i) {
-                Z acc = mk<T>(0, 0);
-                for (int m = 0; m < k; ++m) acc = cfma(from_d2<T>(P->H[i + KLD * m]), dd[m], acc);
-                Np[i + (k + 1) * l] = acc;
-            }
-        }
-    }
+    for (int e = tid; e < k * (k + 1); e += nt) Mp[e] = from_d2<T>(a0.pm->M[e]);
+    for (int e = tid; e < (k + 1) * (k + 1); e += nt) Np[e] = from_d2<T>(a0.pm->N[e]);
     for (int e = tid; e < 2 * nrows; e += nt) {  // x = 0, r = f
         const int b = e / nrows, rr = e - b * nrows;
         xl[b][rr] = mk<T>(0, 0);
@@ -1898,7 +1860,7 @@ mg_status launch_coarse_proj_pair(const CoopArgs<float>& a0in, const CoopArgs<fl
                                   bool* launched) {
     *launched = false;
     CoopArgs<float> a0 = a0in, a1 = a1in;
-    if (a0.A != a1.A || a0.Ah != a1.Ah || a0.W != a1.W || a0.pls != a1.pls || a0.k != a1.k || a0.ms != a1.ms || a0.Nx != a1.Nx ||
+    if (a0.A != a1.A || a0.Ah != a1.Ah || a0.W != a1.W || a0.pm != a1.pm || a0.k != a1.k || a0.ms != a1.ms || a0.Nx != a1.Nx ||
         a0.Nt != a1.Nt || a0.max_cycles != a1.max_cycles) {
         set_error("coarse pair solve: the two solves must share the operator and the deflation space");
         return MG_EINVAL;

@@ -28,7 +28,7 @@ struct CoopArgs {
     C2<T>* r;          // residual workspace
     C2<T>* V;          // Krylov basis, (ms + 1) rows of n
     const C2<T>* W;    // deflation space V_{k+1}, (k + 1) rows of n
-    const KState* pls; // H_k and its QR factorisation
+    const ProjMats* pm;  // projection matrices M, N of the deflation space
     int k, ms;         // deflation size, GMRES cycle length
     double tol;        // stop when ||r|| <= tol ||f||
     int max_cycles;

@@ -162,36 +162,47 @@ __global__ void k_ks_load_dense(KState* ks, const double2* Hk, const double2* ck
     }
 }
 
-__device__ void proj_solve_dev(const KState* pls, const double2* cvec, double2* d, double2* u, double2* g,
-                               double2* ds) {
-    const int lane = threadIdx.x & 31;
-    const int k = pls->j;
-    for (int i = lane; i < KLD; i += 32) g[i] = (i <= k) ? cvec[i] : z0();
+// Column l of M and N (ProjMats) by block l's one warp: M e_l by the stored
+// rotations and a back substitution, N e_l = H_k (M e_l).  Built once per
+// deflation space: the solves that project read the matrices instead of
+// repeating this serial FP64 chain (44 us a cycle in the block solve, and about
+// as long at the start of every coarse cluster kernel in FP64).
+__global__ void k_proj_mats(const KState* pls, ProjMats* pm, int k) {
+    __shared__ double2 g[KLD];
+    __shared__ double2 ds[KMAX];
+    const int lane = threadIdx.x & 31, l = blockIdx.x;
+    for (int i = lane; i < KLD; i += 32) g[i] = (i == l) ? make_double2(1.0, 0.0) : z0();
     __syncwarp();
     if (lane == 0)
         for (int t = 0; t < pls->nrot; ++t) rot_apply(pls->rc[t], pls->rs[t], g[pls->ra[t]], g[pls->rb[t]]);
     __syncwarp();
     solve_upper(pls->R, g, ds, k, nullptr);
     __syncwarp();
-    for (int i = lane; i < k; i += 32) d[i] = ds[i];
+    for (int i = lane; i < k; i += 32) pm->M[i + k * l] = ds[i];
     for (int i = lane; i <= k; i += 32) {
         double2 acc = z0();
-        for (int l = 0; l < k; ++l) acc = cfma(pls->H[i + KLD * l], ds[l], acc);
-        u[i] = acc;
+        for (int m = 0; m < k; ++m) acc = cfma(pls->H[i + KLD * m], ds[m], acc);
+        pm->N[i + (k + 1) * l] = acc;
     }
 }
-__global__ void k_proj_solve(const KState* pls, const double2* cvec, double2* d, double2* u) {
-    __shared__ double2 g[KLD];
-    __shared__ double2 ds[KMAX];
-    proj_solve_dev(pls, cvec, d, u, g, ds);
-}
-__global__ void k_bproj_solve(const KState* pls, const double2* cvec, long cs, double2* d, long dst, double2* u,
-                              long us, Gate act) {
-    __shared__ double2 g[KLD];
-    __shared__ double2 ds[KMAX];
-    const int r = blockIdx.x;
+
+// d = M c and u = N c, one warp per right-hand side
+__global__ void k_bproj_solve(const ProjMats* pm, int k, const double2* cvec, long cs, double2* d, long dst,
+                              double2* u, long us, Gate act) {
+    __shared__ double2 c[KLD];
+    const int r = blockIdx.x, lane = threadIdx.x;
     if (!gate_open(act, r)) return;
-    proj_solve_dev(pls, cvec + r * cs, d + r * dst, u + r * us, g, ds);
+    for (int i = lane; i <= k; i += 32) c[i] = cvec[r * cs + i];
+    __syncwarp();
+    for (int i = lane; i <= k; i += 32) {
+        double2 dv = z0(), uv = z0();
+        for (int l = 0; l <= k; ++l) {
+            if (i < k) dv = cfma(pm->M[i + k * l], c[l], dv);
+            uv = cfma(pm->N[i + (k + 1) * l], c[l], uv);
+        }
+        if (i < k) d[r * dst + i] = dv;
+        u[r * us + i] = uv;
+    }
 }
 
 __global__ void k_set(double* out, double v) {
@@ -603,9 +614,13 @@ void bks_finish(KState* ks, int nb, cudaStream_t s) {
     k_bks_finish<<<nb, 32, 0, s>>>(ks);
     count_launch();
 }
-void bproj_solve(const KState* pls, int nb, const double2* cvec, long cs, double2* d, long ds, double2* u, long us,
-                 Gate act, cudaStream_t s) {
-    k_bproj_solve<<<nb, 32, 0, s>>>(pls, cvec, cs, d, ds, u, us, act);
+void proj_mats(const KState* pls, ProjMats* pm, int k, cudaStream_t s) {
+    k_proj_mats<<<k + 1, 32, 0, s>>>(pls, pm, k);
+    count_launch();
+}
+void bproj_solve(const ProjMats* pm, int k, int nb, const double2* cvec, long cs, double2* d, long ds, double2* u,
+                 long us, Gate act, cudaStream_t s) {
+    k_bproj_solve<<<nb, 32, 0, s>>>(pm, k, cvec, cs, d, ds, u, us, act);
     count_launch();
 }
 void scalar_set(double* out, double v, cudaStream_t s) {
@@ -633,8 +648,8 @@ void ks_load_dense(KState* ks, const double2* Hk, const double2* ck, int k, doub
     k_ks_load_dense<<<1, 32, 0, s>>>(ks, Hk, ck, k, tol_abs);
     count_launch();
 }
-void proj_solve(const KState* pls, const double2* cvec, double2* d, double2* u, cudaStream_t s) {
-    k_proj_solve<<<1, 32, 0, s>>>(pls, cvec, d, u);
+void proj_solve(const ProjMats* pm, int k, const double2* cvec, double2* d, double2* u, cudaStream_t s) {
+    k_bproj_solve<<<1, 32, 0, s>>>(pm, k, cvec, 0, d, 0, u, 0, Gate{});
     count_launch();
 }
 void scalar_rsqrt(double* out, const double* in, cudaStream_t s) {

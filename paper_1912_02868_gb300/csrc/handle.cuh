@@ -152,6 +152,7 @@ struct Handle {
     double2* uvec = nullptr;
     DRState* dr = nullptr;
     KState* pls = nullptr;    // factored H_k of the deflation space
+    ProjMats* pmat = nullptr; // its projection matrices
     double2* cpart = nullptr; // partial sums of the cooperative coarse solve
     int cpart_ctas = 0;
     CoopStats* cstats = nullptr;
@@ -162,6 +163,7 @@ struct Handle {
     double2* fdW = nullptr;   // (k+1) x n0
     KState* fdks = nullptr;
     KState* fdpls = nullptr;
+    ProjMats* fdpmat = nullptr;
     int fine_k = 0;
     // partial intermediate solve
     PartialWS<double> p64;

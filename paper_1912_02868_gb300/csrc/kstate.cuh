@@ -47,6 +47,15 @@ struct DRState {
     int j, k, err;
 };
 
+// The projection of GMRES-Proj onto a deflation space as two matrices, fixed while
+// the space is: d = argmin ||c - H_k d|| = M c and H_k d = N c, with M = R^{-1} Q^+
+// from the factored H_k and N = H_k M.  Column-major, M k x (k + 1) with leading
+// dimension k, N (k + 1) x (k + 1).
+struct ProjMats {
+    double2 M[KMAX * KLD];
+    double2 N[KLD * KLD];
+};
+
 // Start a cycle from a vector of squared norm *nrm2: beta = sqrt(*nrm2),
 // stop when the least-squares residual <= tol_rel * sqrt(*nb2).
 void ks_start(KState* ks, const double* nrm2, double tol_rel, const double* nb2, cudaStream_t s);
@@ -56,9 +65,10 @@ void ks_finish(KState* ks, cudaStream_t s);
 // factor it: the next cycle continues the Arnoldi process from column k.
 // ck == nullptr means c = 0; tol_abs < 0 keeps the state's tolerance.
 void ks_load_dense(KState* ks, const double2* Hk, const double2* ck, int k, double tol_abs, cudaStream_t s);
-// GMRES-Proj least squares with a prepared (ks_load_dense) state:
-// d = argmin ||cvec - H_k d||, u = H_k d.
-void proj_solve(const KState* pls, const double2* cvec, double2* d, double2* u, cudaStream_t s);
+// M and N of a prepared (ks_load_dense) k-column state
+void proj_mats(const KState* pls, ProjMats* pm, int k, cudaStream_t s);
+// GMRES-Proj least squares: d = argmin ||cvec - H_k d||, u = H_k d.
+void proj_solve(const ProjMats* pm, int k, const double2* cvec, double2* d, double2* u, cudaStream_t s);
 // Batched forms over the states ks[0..nb): per right-hand side r the scalars
 // at nrm2[r * ns], nb2[r * nbs], cvec[r * cs], ...; bks_start starts a closed
 // gate's right-hand side as an empty cycle (converged, no steps).
@@ -66,7 +76,7 @@ void bks_start(KState* ks, int nb, const double* nrm2, long ns, double tol_rel, 
                cudaStream_t s);
 void bks_push(KState* ks, int nb, int jh, cudaStream_t s);
 void bks_finish(KState* ks, int nb, cudaStream_t s);
-void bproj_solve(const KState* pls, int nb, const double2* cvec, long cs, double2* d, long ds, double2* u, long us,
+void bproj_solve(const ProjMats* pm, int k, int nb, const double2* cvec, long cs, double2* d, long ds, double2* u, long us,
                  Gate act, cudaStream_t s);
 // strides of KState fields across an array of states, in units of the field's type
 static_assert(sizeof(KState) % sizeof(double2) == 0, "KState arrays are strided in whole double2 units");

@@ -138,9 +138,9 @@ mg_status cg_normal(Handle& H, int l, Level<T>& L, const C2<T>* b, C2<T>* y, C2<
 
 // GMRES-DR(m,k) in FP64 on one grid from x = 0 (Morgan 2002).  V, V2: (m+1) x n
 // bases; the deflation space (V_{k+1}, H_k) of the last cycle is written to Wout
-// and pls (factored), its size to kout.
+// and pls (factored) with its projection matrices pm, its size to kout.
 mg_status dr_solve_on(Handle& H, Level<double>& L, double2* V0, double2* V20, double2* Wout, KState* ks,
-                      KState* pls, int& kout, const double2* f, double2* x, double tol, long long& iters,
+                      KState* pls, ProjMats* pm, int& kout, const double2* f, double2* x, double tol, long long& iters,
                       cudaStream_t s) {
     const long n = L.n;
     const int m = H.p.dr_m, k = H.p.dr_k;
@@ -211,6 +211,7 @@ mg_status dr_solve_on(Handle& H, Level<double>& L, double2* V0, double2* V20, do
                 set_error("GMRES-DR produced no deflation space");
                 return MG_ECUDA;
             }
+            proj_mats(pls, pm, kout, s);
             return MG_OK;
         }
         std::swap(V, V2);
@@ -232,7 +233,7 @@ double coarse_tol_proj(const Handle& H) {
 // deflation space of the handle.
 mg_status dr_solve(Handle& H, const double2* f, double2* x, cudaStream_t s) {
     long long iters = 0;
-    MG_TRY(dr_solve_on(H, H.L64[2], H.c64.V, H.c64.V2, H.c64.W, H.c64.ks, H.pls, H.defl_k, f, x,
+    MG_TRY(dr_solve_on(H, H.L64[2], H.c64.V, H.c64.V2, H.c64.W, H.c64.ks, H.pls, H.pmat, H.defl_k, f, x,
                        coarse_tol_dr(H), iters, s));
     H.st.coarse_iters += iters;
     H.st.mvps[2] += iters;
@@ -244,7 +245,7 @@ mg_status dr_solve(Handle& H, const double2* f, double2* x, cudaStream_t s) {
 // (used by the fine-grid deflation arm): minimum-residual projection onto
 // (W = V_{k+1}, H_k), then one GMRES(m - k) cycle, repeated.
 mg_status proj_solve_host(Handle& H, Level<double>& L, double2* V, const double2* W, double2* r, KState* ks,
-                          const KState* pls, int k, const double2* f, double2* x, double tol, long long& iters,
+                          const ProjMats* pm, int k, const double2* f, double2* x, double tol, long long& iters,
                           cudaStream_t s) {
     const long n = L.n;
     const int ms = std::max(H.p.dr_m - k, 1);
@@ -257,7 +258,7 @@ mg_status proj_solve_host(Handle& H, Level<double>& L, double2* V, const double2
     iters = 0;
     while (true) {
         launch_gram<double>(H.cvec, W, n, k + 1, r, n, H.red, Gate{}, s);
-        proj_solve(pls, H.cvec, H.dvec, H.uvec, s);
+        proj_solve(pm, k, H.cvec, H.dvec, H.uvec, s);
         launch_axpy_multi<double>(x, W, n, k, nullptr, H.dvec, 1.0, false, n, nullptr, H.red, Gate{}, s);
         launch_axpy_multi<double>(r, W, n, k + 1, nullptr, H.uvec, -1.0, false, n, r2, H.red, Gate{}, s);
         ks_start(ks, r2, tol, nb2, s);
@@ -298,7 +299,7 @@ CoopArgs<T> proj_args(Handle& H, const C2<T>* f, C2<T>* x) {
     a.r = W.r;
     a.V = W.V;
     a.W = W.W;
-    a.pls = H.pls;
+    a.pm = H.pmat;
     a.k = H.defl_k;
     a.ms = std::max(H.p.dr_m - H.defl_k, 1);
     a.tol = coarse_tol_proj(H);
@@ -711,10 +712,10 @@ mg_status fine_deflated_solve(Handle& H, const double2* b, double2* x, double to
     const long n = L0.n;
     long long it = 0;
     if (H.fine_k == 0) {
-        MG_TRY(dr_solve_on(H, L0, H.fdV, H.fdV2, H.fdW, H.fdks, H.fdpls, H.fine_k, b, x, tol, it, s));
+        MG_TRY(dr_solve_on(H, L0, H.fdV, H.fdV2, H.fdW, H.fdks, H.fdpls, H.fdpmat, H.fine_k, b, x, tol, it, s));
         H.st.dr_solves += 1;
     } else {
-        MG_TRY(proj_solve_host(H, L0, H.fdV, H.fdW, H.fr, H.fdks, H.fdpls, H.fine_k, b, x, tol, it, s));
+        MG_TRY(proj_solve_host(H, L0, H.fdV, H.fdW, H.fr, H.fdks, H.fdpmat, H.fine_k, b, x, tol, it, s));
     }
     H.st.mvps[0] += it + 1;
     double* fnb2 = MG_DEVF(H.sc, double, tmp) + 4;

@@ -314,7 +314,7 @@ mg_status bcoarse_proj(Handle& H, const float2* f, float2* x, int nb, Gate act, 
     // right-hand side, so the same sequence serves every cycle
     auto cycle = [&](cudaStream_t cs) {
         launch_bgram<float>(B.cg, KLD, W, n, 0, k + 1, nullptr, 0, B.cr, n, n, nb, B.red, ca, cs);
-        bproj_solve(H.pls, nb, B.cg, KLD, B.cd, KLD, B.cu, KLD, ca, cs);
+        bproj_solve(H.pmat, k, nb, B.cg, KLD, B.cd, KLD, B.cu, KLD, ca, cs);
         launch_baxpy<float>(x, n, W, n, 0, k, nullptr, 0, B.cd, KLD, 1.0, false, n, nb, nullptr, 0, B.red, ca, cs);
         launch_baxpy<float>(B.cr, n, W, n, 0, k + 1, nullptr, 0, B.cu, KLD, -1.0, false, n, nb, cr2, NSC, B.red, ca,
                             cs);
