@@ -44,38 +44,25 @@
 #include <type_traits>
 #include <vector>
 
-#include "coarse_coop.cuh"
+#include "coarse_dev.cuh"
 
 namespace cg = cooperative_groups;
 
 namespace mg {
 
+using namespace cdev;
+
 namespace {
 
-constexpr int NDOF = 24;
 constexpr int MAX_THREADS = 512;
 constexpr int MAX_SPC = 16;       // sites per apply chunk (staged neighbour rows)
 constexpr int MAX_NB_SITES = 64;  // sites per CTA in the neighbour table
-constexpr int MAX_CLUSTER = 16;    // CTAs of one cluster (non-portable size)
-constexpr size_t SMEM_LIMIT = 227 * 1024;
-constexpr long FLOW_SPIN = 1L << 20;  // default try_wait rounds before a dataflow wait gives up
 // FP16 operator (push mode): the blocks of directions 0..ASH_DIRS-1 of a CTA's
 // sites stay in its shared memory for the whole solve, the other directions
 // stream from L2 each step.  A site's part is padded by 24 words so that the two
 // sites one warp reads fall on different banks.
 constexpr int ASH_DIRS = 3;
 constexpr int ASH_SITE_WORDS = ASH_DIRS * 24 * 24 + 24;
-
-template <typename R>
-struct Small {  // per-CTA copy of the small least-squares state, precision R
-    using Z = C2<R>;
-    Z H[(MSMAX + 1) * MSMAX];  // column-major, ld MSMAX + 1 (unrotated)
-    Z Rm[(MSMAX + 1) * MSMAX];
-    R rc[MSMAX];
-    Z rs[MSMAX];
-    Z g[MSMAX + 1], c[MSMAX + 1], d[MSMAX], rho[MSMAX + 1];
-    Z pd[KMAX], pu[KLD];       // projection coefficients
-};
 
 template <typename T>
 struct ClusterSmem {
@@ -111,85 +98,6 @@ __host__ __device__ inline size_t proj_bytes(int k) {
     return (size_t)(k * (k + 1) + (k + 1) * (k + 1)) * sizeof(C2<T>);
 }
 
-template <typename R>
-__device__ __forceinline__ R cabs_(C2<R> a) { return sqrt(a.x * a.x + a.y * a.y); }
-
-template <typename R>
-__device__ __forceinline__ C2<R> cdiv_(C2<R> a, C2<R> b) {
-    if (fabs(b.x) >= fabs(b.y)) {
-        R r = b.y / b.x, den = b.x + b.y * r;
-        return mk<R>((a.x + a.y * r) / den, (a.y - a.x * r) / den);
-    }
-    R r = b.x / b.y, den = b.x * r + b.y;
-    return mk<R>((a.x * r + a.y) / den, (a.y * r - a.x) / den);
-}
-
-// acc - a * b with every rounding step fixed: both cluster kernels get the same
-// operations, whatever contraction the compiler would pick for a * b - c * d
-template <typename R>
-__device__ __forceinline__ C2<R> cfms_(C2<R> a, C2<R> b, C2<R> acc) {
-    acc.x = fma(-a.x, b.x, acc.x);
-    acc.x = fma(a.y, b.y, acc.x);
-    acc.y = fma(-a.x, b.y, acc.y);
-    acc.y = fma(-a.y, b.x, acc.y);
-    return acc;
-}
-
-// d = R^{-1} g for the jc x jc upper-triangular R (column-major, leading
-// dimension MSMAX + 1, jc <= MSMAX < 32) by one warp, column by column. The
-// lanes first form the reciprocals of their pivots at once (a zero pivot gives
-// zero, so d_i = 0 there); then lane i keeps g_i minus the columns already
-// eliminated, and in turn i its d_i = (that) / R_ii is broadcast to the lanes
-// above.  Only a product, a shuffle and a subtraction stay on the serial chain.
-template <typename R>
-__device__ __forceinline__ void back_subst_warp(const C2<R>* Rm, const C2<R>* g, C2<R>* d, int jc, int lane) {
-    constexpr int LDR = MSMAX + 1;
-    C2<R> inv = mk<R>(0, 0), acc = mk<R>(0, 0);
-    if (lane < jc) {
-        const C2<R> piv = Rm[lane + LDR * lane];
-        if (piv.x != R(0) || piv.y != R(0)) inv = cdiv_<R>(mk<R>(1, 0), piv);
-        acc = g[lane];
-    }
-    for (int i = jc - 1; i >= 0; --i) {
-        const C2<R> rli = (lane < i) ? Rm[lane + LDR * i] : mk<R>(0, 0);
-        C2<R> di = mk<R>(fma(-acc.y, inv.y, acc.x * inv.x), fma(acc.y, inv.x, acc.x * inv.y));
-        di.x = __shfl_sync(0xffffffffu, di.x, i);
-        di.y = __shfl_sync(0xffffffffu, di.y, i);
-        if (lane == i) d[i] = di;
-        if (lane < i) acc = cfms_<R>(rli, di, acc);
-    }
-}
-
-template <typename R>
-__device__ __forceinline__ R rsqrt_(R x) {
-    if constexpr (std::is_same<R, float>::value)
-        return rsqrtf(x);
-    else
-        return rsqrt(x);
-}
-
-// Complex Givens rotation G = [[c, s], [-conj(s), c]] with G [a; h] = [r; 0]
-// for a real, non-negative h (the new subdiagonal entry).
-template <typename R>
-__device__ __forceinline__ void givens_real_(C2<R> a, R h, R& c, C2<R>& s, C2<R>& r) {
-    if (h == R(0)) { c = R(1); s = mk<R>(0, 0); r = a; return; }
-    const R aa2 = a.x * a.x + a.y * a.y;
-    if (aa2 == R(0)) { c = R(0); s = mk<R>(1, 0); r = mk<R>(h, 0); return; }
-    // reciprocal square roots only: no divide on this serial path
-    const R rh2 = aa2 + h * h;
-    const R inv_aa = rsqrt_(aa2), inv_rh = rsqrt_(rh2);
-    c = aa2 * inv_aa * inv_rh;
-    const C2<R> ph = mk<R>(a.x * inv_aa, a.y * inv_aa);
-    s = cscale(ph, h * inv_rh);
-    r = cscale(ph, rh2 * inv_rh);
-}
-template <typename R>
-__device__ __forceinline__ void rot_(R c, C2<R> s, C2<R>& up, C2<R>& uq) {
-    const C2<R> p = up, q = uq;
-    up = cadd(cscale(p, c), cmul(s, q));
-    uq = csub(cscale(q, c), cmul(conj_(s), p));
-}
-
 // One complex entry of the FP16 operator copy (real part in the low half)
 template <typename T>
 __device__ __forceinline__ C2<T> half_bits(unsigned u) {
@@ -199,137 +107,6 @@ __device__ __forceinline__ C2<T> half_bits(unsigned u) {
 template <typename T>
 __device__ __forceinline__ C2<T> half_entry(const unsigned* p) {
     return half_bits<T>(__ldg(p));
-}
-
-// ---- tensor-core apply of the FP16 operator (a.mma) ----
-// The staged vector holds each complex entry x as two FP16 pairs: hi = (Re, Im)
-// of x 2^10 rounded to FP16, lo = the same of the remainder, in the two words of
-// one 8-byte slot.  2^10 keeps both parts normal for the entries of a unit
-// vector and leaves a factor 64 below the FP16 range; hi + lo carries 22 bits.
-constexpr float TC_XS = 1024.f;
-constexpr float TC_XS_INV = 1.f / 1024.f;
-
-__device__ __forceinline__ float2 tc_split(float2 v) {
-    const __half2 hi = __floats2half2_rn(v.x * TC_XS, v.y * TC_XS);
-    const float2 hf = __half22float2(hi);
-    // v 2^10 - hi is exact in FP32 (hi is v 2^10 rounded to 11 bits)
-    const __half2 lo = __floats2half2_rn(fmaf(v.x, TC_XS, -hf.x), fmaf(v.y, TC_XS, -hf.y));
-    return make_float2(__uint_as_float(*reinterpret_cast<const unsigned*>(&hi)),
-                       __uint_as_float(*reinterpret_cast<const unsigned*>(&lo)));
-}
-template <typename T>
-__device__ __forceinline__ C2<T> stage_value(C2<T> v, bool split) {
-    if constexpr (std::is_same<T, float>::value) return split ? tc_split(v) : v;
-    return v;
-}
-
-// Word of the B fragment that lane column n = g (0..7) takes from a staged entry
-// p (rows 2l, 2l + 1 of the real form): n = 0: (Re hi, -Im hi), 1: (Im hi, Re hi),
-// 2 and 3: the same of lo, 4..7: zero.  The low half is the lower row.
-__device__ __forceinline__ unsigned tc_bword(float2 p, int g) {
-    const unsigned src = __float_as_uint((g & 2) ? p.y : p.x);
-    const unsigned w = (g & 1) ? __byte_perm(src, 0u, 0x1032) : (src ^ 0x80000000u);
-    return g < 4 ? w : 0u;
-}
-
-__device__ __forceinline__ void tc_mma(float (&c)[4], unsigned a0, unsigned a1, unsigned a2, unsigned a3, unsigned b0,
-                                       unsigned b1) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
-        "{%0, %1, %2, %3};\n"
-        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
-// w = sum_d A_d x_d for one own site on tensor cores (m16n8k16, FP16 inputs,
-// FP32 accumulation), by one whole warp.  Each complex product is the real
-// product A'' B'': A'' (24 x 48) has Re and Im of column l of A_d in columns
-// 2l and 2l + 1, so a stored FP16 word (real part in the low half) is already
-// an element pair of an A fragment; B'' (48 x 8) holds in rows 2l, 2l + 1 the
-// pairs of tc_bword for the staged x_d[l].  Then Re w = (column 0 + column 2)
-// 2^-10 and Im w = (column 1 + column 3) 2^-10.  The 24 rows are two M tiles,
-// the second with rows 24..31 zero; the 5 directions x 24 columns are 15 K
-// tiles.  Blocks are column-major: entry (row i, column l) of direction d is
-// word (d 24 + l) 24 + i.  Directions < ASH_DIRS come from shared memory, the
-// others from the FP16 operator in global memory, whose fragments
-// (tc_load_stream) are loaded first, so that their latency overlaps the
-// shared-memory directions, which every site accumulates first.
-constexpr int TC_SW = (5 - ASH_DIRS) * 3 * 6;  // stream fragment words a lane holds for one site
-struct TcAcc {
-    float m0[4], m1[4];  // M tiles 0 (rows 0..15) and 1 (rows 16..23)
-};
-__device__ __forceinline__ void tc_zero(TcAcc& c) {
-#pragma unroll
-    for (int u = 0; u < 4; ++u) c.m0[u] = c.m1[u] = 0.f;
-}
-// the A fragments of direction d, K tile kt from a site's blocks p (lane offset applied)
-__device__ __forceinline__ void tc_frag(const unsigned* p, unsigned (&q)[6]) {
-    q[0] = p[0];
-    q[1] = p[8];
-    q[2] = p[4 * NDOF];
-    q[3] = p[4 * NDOF + 8];
-    q[4] = p[16];
-    q[5] = p[4 * NDOF + 16];
-}
-__device__ __forceinline__ void tc_step(TcAcc& c, const unsigned (&q)[6], float2 x0, float2 x1, int g) {
-    const unsigned b0 = tc_bword(x0, g), b1 = tc_bword(x1, g);
-    tc_mma(c.m0, q[0], q[1], q[2], q[3], b0, b1);
-    tc_mma(c.m1, q[4], 0u, q[5], 0u, b0, b1);
-}
-// fragments of the streamed directions of one site (Ag: the site's blocks)
-__device__ __forceinline__ void tc_load_stream(const unsigned* __restrict__ Ag, unsigned (&f)[TC_SW], int lane) {
-    const int g = lane >> 2, t = lane & 3;
-#pragma unroll
-    for (int d = ASH_DIRS; d < 5; ++d)
-#pragma unroll
-        for (int kt = 0; kt < 3; ++kt) {
-            const unsigned* p = Ag + (d * NDOF + 8 * kt + t) * NDOF + g;
-            unsigned* q = f + ((d - ASH_DIRS) * 3 + kt) * 6;
-            q[0] = __ldg(p);
-            q[1] = __ldg(p + 8);
-            q[2] = __ldg(p + 4 * NDOF);
-            q[3] = __ldg(p + 4 * NDOF + 8);
-            q[4] = __ldg(p + 16);
-            q[5] = __ldg(p + 4 * NDOF + 16);
-        }
-}
-__device__ __forceinline__ void tc_stream_dirs(TcAcc& c, const unsigned (&f)[TC_SW], const float2 (*xs)[NDOF],
-                                               int lane) {
-    const int g = lane >> 2, t = lane & 3;
-#pragma unroll
-    for (int d = ASH_DIRS; d < 5; ++d)
-#pragma unroll
-        for (int kt = 0; kt < 3; ++kt) {
-            unsigned q[6];
-#pragma unroll
-            for (int u = 0; u < 6; ++u) q[u] = f[((d - ASH_DIRS) * 3 + kt) * 6 + u];
-            tc_step(c, q, xs[d][8 * kt + t], xs[d][8 * kt + t + 4], g);
-        }
-}
-// As: the site's shared-memory blocks
-__device__ __forceinline__ void tc_shared_dirs(TcAcc& c, const unsigned* As, const float2 (*xs)[NDOF], int lane) {
-    const int g = lane >> 2, t = lane & 3;
-#pragma unroll
-    for (int d = 0; d < ASH_DIRS; ++d)
-#pragma unroll
-        for (int kt = 0; kt < 3; ++kt) {
-            unsigned q[6];
-            tc_frag(As + (d * NDOF + 8 * kt + t) * NDOF + g, q);
-            tc_step(c, q, xs[d][8 * kt + t], xs[d][8 * kt + t + 4], g);
-        }
-}
-// out[0..23] = c 2^-10: lane t = 0 holds columns 0, 1 (hi) and lane t = 1
-// columns 2, 3 (lo) of rows g, g + 8 (M tile 0) and 16 + g (M tile 1)
-__device__ __forceinline__ void tc_store(const TcAcc& c, float2* out, int lane) {
-    const int g = lane >> 2, t = lane & 3;
-    float r[6] = {c.m0[0], c.m0[1], c.m0[2], c.m0[3], c.m1[0], c.m1[1]};
-#pragma unroll
-    for (int u = 0; u < 6; ++u) r[u] += __shfl_xor_sync(0xffffffffu, r[u], 1);
-    if (t == 0) {
-        out[g] = make_float2(r[0] * TC_XS_INV, r[1] * TC_XS_INV);
-        out[g + 8] = make_float2(r[2] * TC_XS_INV, r[3] * TC_XS_INV);
-        out[g + 16] = make_float2(r[4] * TC_XS_INV, r[5] * TC_XS_INV);
-    }
 }
 
 // Store v at the address dst has in the shared memory of CTA `rank` of the
@@ -456,80 +233,15 @@ __device__ void reduce_inbox(const C2<T>* inbox, int nr, int n, C2<T>* red, int 
     __syncthreads();
 }
 
-// Split cluster barrier: arrive (releasing this thread's writes, shared and
-// global, to the cluster) and wait (acquiring everyone's).  Work placed between
-// the two overlaps the barrier's latency.  Every thread of a warp executes both.
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); }
-
-// Dataflow exchange (push mode): instead of a cluster barrier after each push,
-// every value goes out by st.async, which counts its bytes on an mbarrier in the
-// receiving CTA; a CTA goes on once its barrier has seen all the bytes of the
-// phase (armed by its thread 0 with the expected count).
-__device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ unsigned cluster_addr(unsigned local, int rank) {
-    unsigned r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(local), "r"(rank));
-    return r;
-}
-__device__ __forceinline__ void mbar_init(unsigned long long* bar, unsigned count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_addr(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arm(unsigned long long* bar, unsigned bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_addr(bar)), "r"(bytes)
-                 : "memory");
-}
-// bounded wait for the completion of the phase with this parity (acquiring the
-// cluster's st.async writes); false when it gave up
-__device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned parity, long spin) {
-    const unsigned addr = smem_addr(bar);
-    for (long it = 0; it < spin; ++it) {
-        unsigned ok;
-        asm volatile(
-            "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
-            " selp.u32 %0, 1, 0, p;\n}\n"
-            : "=r"(ok)
-            : "r"(addr), "r"(parity)
-            : "memory");
-        if (ok) return true;
-    }
-    return false;
-}
-// barrier 1 over the first nthreads threads (the row warps)
-__device__ __forceinline__ void row_warps_sync(int nthreads) {
-    asm volatile("bar.sync 1, %0;\n" ::"r"(nthreads) : "memory");
-}
-__device__ __forceinline__ void st_async(unsigned dst, float2 v, unsigned bar) {
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];\n" ::"r"(dst),
-                 "f"(v.x), "f"(v.y), "r"(bar)
-                 : "memory");
-}
-__device__ __forceinline__ void st_async(unsigned dst, double2 v, unsigned bar) {
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f64 [%0], {%1, %2}, [%3];\n" ::"r"(dst),
-                 "d"(v.x), "d"(v.y), "r"(bar)
-                 : "memory");
-}
-
-__device__ __forceinline__ long nbr_site(long s, int d, int Nx, int Nt) {
-    const int xx = (int)(s % Nx), tt = (int)(s / Nx);
-    if (d == 1) return (xx + 1 == Nx) ? s - xx : s + 1;
-    if (d == 2) return (xx == 0) ? s + Nx - 1 : s - 1;
-    if (d == 3) return (tt + 1 == Nt) ? (long)xx : s + Nx;
-    if (d == 4) return (tt == 0) ? s + (long)Nx * (Nt - 1) : s - Nx;
-    return s;
-}
-
 // Write element k of own row (site ls) of a new basis vector into the five
-// staging slots that read it (push mode); split: as the tensor-core apply's
-// two FP16 parts (tc_split).
+// staging slots that read it (push mode).
 template <typename T>
-__device__ __forceinline__ void push_row(ClusterSmem<T>& S, int me, int e, C2<T> v, bool split) {
+__device__ __forceinline__ void push_row(ClusterSmem<T>& S, int me, int e, C2<T> v) {
     const int ls = e / NDOF, kk = e - ls * NDOF;
-    const C2<T> sv = stage_value<T>(v, split);
 #pragma unroll
     for (int q = 0; q < 5; ++q) {
         const int code = S.pusht[ls][q];
-        st_rank<T>(&S.xs[(code >> 3) & 0x1fff][code & 7][kk], code >> 16, me, sv);
+        st_rank<T>(&S.xs[(code >> 3) & 0x1fff][code & 7][kk], code >> 16, me, v);
     }
 }
 
@@ -570,14 +282,13 @@ __device__ void push_gram_flow(const C2<T>* X, long ldx, int nd, const C2<T>* y,
     }
 }
 template <typename T>
-__device__ __forceinline__ void push_row_flow(ClusterSmem<T>& S, int e, C2<T> v, bool split) {
+__device__ __forceinline__ void push_row_flow(ClusterSmem<T>& S, int e, C2<T> v) {
     const int ls = e / NDOF, kk = e - ls * NDOF;
     const unsigned bar = smem_addr(&S.mb[2]);
-    const C2<T> sv = stage_value<T>(v, split);
 #pragma unroll
     for (int q = 0; q < 5; ++q) {
         const int code = S.pusht[ls][q], owner = code >> 16;
-        st_async(cluster_addr(smem_addr(&S.xs[(code >> 3) & 0x1fff][code & 7][kk]), owner), sv,
+        st_async(cluster_addr(smem_addr(&S.xs[(code >> 3) & 0x1fff][code & 7][kk]), owner), v,
                  cluster_addr(bar, owner));
     }
 }
@@ -659,10 +370,6 @@ __global__ void __maxnreg__(128) k_coarse_proj(CoopArgs<T> a) {
     // received this CTA's contribution to a later exchange, which this CTA makes
     // after it has read the buffer.
     const bool flow = push && a.flow;
-    // tensor-core apply (tc_apply_site): FP32 dataflow mode with the FP16 operator,
-    // its first directions in shared memory, and CGS2; the staging slots then hold
-    // split values
-    const bool mma = std::is_same<T, float>::value && flow && a.ash && a.mma && !a.dc;
 #ifdef CP_PHASE_CLOCKS
     const bool clk = rank == 0 && tid == 0 && atomicAdd(&cp_clock_launches, 1u) < 48u;
     long long acc_t[7] = {0, 0, 0, 0, 0, 0, 0}, t_prev = clock64();
@@ -867,7 +574,7 @@ __global__ void __maxnreg__(128) k_coarse_proj(CoopArgs<T> a) {
             for (int e = tid; e < nrows; e += nt) {
                 const Z v = accum_rows<T, true>(w[e], Vl, ldv, e, S.h1, 1);
                 w[e] = v;
-                push_row_flow<T>(S, e, v, mma);
+                push_row_flow<T>(S, e, v);
             }
         }
         for (int j = 1; j < ms; ++j) {
@@ -920,7 +627,7 @@ __global__ void __maxnreg__(128) k_coarse_proj(CoopArgs<T> a) {
                 for (int e = tid; e < nrows; e += nwr * 32) {  // row warps only
                     const Z v = cscale(accum_rows<T, true>(wl[e], Vl, ldv, e, S.zc, j + 1), irho);
                     wl[e] = v;
-                    push_row_flow<T>(S, e, v, mma);
+                    push_row_flow<T>(S, e, v);
                 }
             }
             ++iters;
@@ -1022,7 +729,7 @@ __global__ void __maxnreg__(128) k_coarse_proj(CoopArgs<T> a) {
                 const Z v = cscale(rl[e], sc);
                 Vl[e] = v;
                 if (push)
-                    push_row<T>(S, rank, e, v, mma);
+                    push_row<T>(S, rank, e, v);
                 else if (a.vs)
                     a.V[r0 + e] = v;
             }
@@ -1050,23 +757,7 @@ __global__ void __maxnreg__(128) k_coarse_proj(CoopArgs<T> a) {
                     }
                     __syncthreads();
                 }
-                if (mma) {  // push mode: c0 == 0, cs == my_sites
-                    if constexpr (std::is_same<T, float>::value) {
-                        // one site per row warp at a time; its streamed fragments are
-                        // loaded first and arrive during the shared-memory directions
-                        const int lane = tid & 31;
-                        if ((tid >> 5) < nwr)
-                            for (int ls = tid >> 5; ls < cs; ls += nwr) {
-                                unsigned f[TC_SW];
-                                tc_load_stream(a.Ah + (s0 + ls) * (5L * NDOF * NDOF), f, lane);
-                                TcAcc c;
-                                tc_zero(c);
-                                tc_shared_dirs(c, Ash + ls * ASH_SITE_WORDS, S.xs[ls], lane);
-                                tc_stream_dirs(c, f, S.xs[ls], lane);
-                                tc_store(c, wl + (long)ls * NDOF, lane);
-                            }
-                    }
-                } else if (a.Ah) {  // FP16 operator copy: half the bytes of the stream, FP32 arithmetic
+                if (a.Ah) {  // FP16 operator copy: half the bytes of the stream, FP32 arithmetic
                     for (int e = tid; e < cs * NDOF; e += nt) {
                         const int ls = e / NDOF, kk = e - ls * NDOF;
                         const unsigned* Ab = a.Ah + (s0 + c0 + ls) * (5L * NDOF * NDOF) + kk;
@@ -1151,9 +842,9 @@ __global__ void __maxnreg__(128) k_coarse_proj(CoopArgs<T> a) {
                     const Z v = cscale(accum_rows<T, true>(wl[e], Vl, ldv, e, S.red, j + 1), sc);
                     wl[e] = v;
                     if (flow)
-                        push_row_flow<T>(S, e, v, mma);
+                        push_row_flow<T>(S, e, v);
                     else if (push)
-                        push_row<T>(S, rank, e, v, mma);
+                        push_row<T>(S, rank, e, v);
                     else if (a.vs)
                         wg[e] = v;
                 }
@@ -1225,13 +916,13 @@ __global__ void __maxnreg__(128) k_coarse_proj(CoopArgs<T> a) {
         a.out->ash = a.ash;
         a.out->half = a.Ah ? 1 : 0;
         a.out->paired = 0;
-        a.out->mma = mma ? 1 : 0;
+        a.out->mma = 0;
     }
 #ifdef CP_PHASE_CLOCKS
     if (clk && clk_steps > 0)
-        printf("coarse_proj phases (cycles/step over %d steps, mma %d): staging wait %lld, apply %lld, gram1+wait %lld, "
+        printf("coarse_proj phases (cycles/step over %d steps): staging wait %lld, apply %lld, gram1+wait %lld, "
                "reduce+update %lld, gram2+wait %lld, reduce+v+push %lld, other %lld\n",
-               clk_steps, mma ? 1 : 0, acc_t[0] / clk_steps, acc_t[1] / clk_steps, acc_t[2] / clk_steps,
+               clk_steps, acc_t[0] / clk_steps, acc_t[1] / clk_steps, acc_t[2] / clk_steps,
                acc_t[3] / clk_steps, acc_t[4] / clk_steps, acc_t[5] / clk_steps, acc_t[6] / clk_steps);
 #endif
     cluster.sync();  // no CTA leaves while others may still read its shared memory
@@ -1825,6 +1516,12 @@ mg_status geometry(long nsite, int ms, int k, Geometry& g) {
 template <typename T>
 mg_status launch_coarse_proj(const CoopArgs<T>& args_in, cudaStream_t s) {
     CoopArgs<T> a = args_in;
+    if constexpr (std::is_same<T, float>::value) {
+        // the FP16 operator on tensor cores, basis and operator on chip (coarse_tc.cu)
+        bool done = false;
+        if (a.ms >= 1 && a.ms <= MSMAX && a.k >= 1 && a.k + 1 <= PSTR) MG_TRY(launch_coarse_tc(a, s, &done));
+        if (done) return MG_OK;
+    }
     if (a.ms < 1 || a.ms > MSMAX || a.k < 1 || a.k + 1 > PSTR || a.ms + 2 > PSTR) {
         set_error("coarse solve: unsupported (m - k, k) = (%d, %d)", a.ms, a.k);
         return MG_EINVAL;

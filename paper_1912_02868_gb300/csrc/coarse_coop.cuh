@@ -46,13 +46,18 @@ struct CoopArgs {
     long spin;         // try_wait rounds before a dataflow wait gives up (0: the default, 2^20)
     int probe;         // 1 (tests): before the first cycle every row thread waits, bounded by
                        // `spin`, on a barrier that nothing completes, so the give-up path runs
-    int mma;           // 1: the apply runs on tensor cores where the kernel can (FP32 dataflow mode
-                       // with the FP16 blocks in shared memory, CGS2): FP16 operator times the
-                       // vector split into two FP16 parts, FP32 accumulation
+    int mma;           // 1: the apply runs on tensor cores where it can (coarse_tc.cu: FP32 vectors,
+                       // at most 16 sites a CTA, CGS2): FP16 operator times the vector split into
+                       // two FP16 parts, FP32 accumulation
 };
 
 template <typename T>
 mg_status launch_coarse_proj(const CoopArgs<T>& a, cudaStream_t s);
+
+// The same solve with the FP16 operator applied on tensor cores (coarse_tc.cu);
+// *launched is false (and nothing is enqueued) where that kernel does not serve
+// the arguments.
+mg_status launch_coarse_tc(const CoopArgs<float>& a, cudaStream_t s, bool* launched);
 
 // The projected solves of two right-hand sides of one coarsest operator (same
 // A, deflation space and parameters; own f, x, r, V and counters) in one
