@@ -55,6 +55,14 @@ mg_status halloc(Handle& H, void** p, size_t bytes) {
     return MG_OK;
 }
 
+mg_status clear_coarse_exchange(Handle& H, cudaStream_t s) {
+    if (!H.cpart) return MG_OK;
+    MG_CUDA_TRY(cudaMemsetAsync(H.cpart, 0, (size_t)2 * H.cpart_ctas * PSTR * sizeof(double2), s));
+    MG_CUDA_TRY(cudaMemsetAsync(H.crows, 0, (size_t)2 * H.L64[2].n * sizeof(double2), s));
+    MG_CUDA_TRY(cudaMemsetAsync(H.cepoch, 0, sizeof(unsigned), s));
+    return MG_OK;
+}
+
 template <typename T> mg_status vcycle_entry(Handle& H, const C2<T>* f, C2<T>* x, cudaStream_t s);
 
 namespace {
@@ -193,8 +201,13 @@ mg_status alloc_workspaces(Handle& H, cudaStream_t s, bool owner) {
     MG_TRY(halloc_t(H, &H.dr, 1));
     if (owner) MG_TRY(halloc_t(H, &H.pls, 1));
     if (owner) MG_TRY(halloc_t(H, &H.pmat, 1));
-    H.cpart_ctas = sm_count();
-    MG_TRY(halloc_t(H, &H.cpart, (size_t)2 * H.cpart_ctas * PSTR));
+    if (p.precision != MG_FP64 && p.coarse_half && (long)H.L64[2].Nx * H.L64[2].Nt > 256) {
+        H.cpart_ctas = sm_count();
+        MG_TRY(halloc_t(H, &H.cpart, (size_t)2 * H.cpart_ctas * PSTR));
+        MG_TRY(halloc_t(H, &H.crows, (size_t)2 * n2));
+        MG_TRY(halloc_t(H, &H.cepoch, 1));
+        MG_TRY(clear_coarse_exchange(H, s));
+    }
     MG_TRY(halloc_t(H, &H.cstats, 1));
     if (p.partial_tol > 0.0) {
         const long n1 = H.L64[1].n;
@@ -267,7 +280,10 @@ mg_status solve_rhs_pairs(Handle& A, Handle& Bh, const double2* B, double2* X, i
         std::memcpy(&cs, Hp->pinned, sizeof cs);
         Hp->st.coarse_iters += cs.iters;
         Hp->st.mvps[2] += cs.iters;
-        if (cs.timeouts) return set_error("coarse solve: a bounded wait of the dataflow exchange gave up"), MG_ETIMEOUT;
+        if (cs.timeouts) {
+            MG_TRY(clear_coarse_exchange(*Hp, s));
+            return set_error("coarse solve: a bounded wait of the dataflow exchange gave up"), MG_ETIMEOUT;
+        }
     }
     return result;
 }
@@ -315,7 +331,10 @@ mg_status solve_rhs(Handle& H, const double2* B, double2* X, bool bdev, bool xde
     std::memcpy(&cs, H.pinned, sizeof cs);
     H.st.coarse_iters += cs.iters;
     H.st.mvps[2] += cs.iters;
-    if (cs.timeouts) return set_error("coarse solve: a bounded wait of the dataflow exchange gave up"), MG_ETIMEOUT;
+    if (cs.timeouts) {
+        MG_TRY(clear_coarse_exchange(H, s));
+        return set_error("coarse solve: a bounded wait of the dataflow exchange gave up"), MG_ETIMEOUT;
+    }
     return result;
 }
 

@@ -43,6 +43,8 @@ CoopArgs<T> coarse_args(Handle& H, const C2<T>* f, C2<T>* x, C2<T>* r, C2<T>* V,
     a.max_cycles = H.p.proj_max_cycles;
     a.part = part;
     a.part_ctas = part_ctas;
+    a.rows = H.crows;
+    a.epoch = H.cepoch;
     a.out = out;
     a.Ah = std::is_same<T, float>::value ? H.A16c : nullptr;
     a.dc = H.p.coarse_dcgs2;
@@ -176,6 +178,8 @@ mg_status mg_coarse_solve(mg_handle h, int precision, int nrhs, const void* b, v
         info->cycles = cs[0].cycles;
         info->timeouts = timeouts;
     }
+    if (timeouts)
+        for (int r = 0; r < nrhs; ++r) MG_TRY(clear_coarse_exchange(*HH[r], s));
     if (timeouts) return set_error("coarse solve: a bounded wait of the dataflow exchange gave up"), MG_ETIMEOUT;
     return MG_OK;
 }

@@ -32,14 +32,19 @@ struct CoopArgs {
     int k, ms;         // deflation size, GMRES cycle length
     double tol;        // stop when ||r|| <= tol ||f||
     int max_cycles;
-    double2* part;     // partial sums: 2 x part_ctas x PSTR
+    // exchange buffers of the grid form of coarse_tc.cu (null: not allocated): tagged
+    // partial sums (2 x PSTR x part_ctas), tagged rows (2 x n) and the launch's tag base
+    double2* part;
     int part_ctas;
+    double2* rows;
+    unsigned* epoch;
     CoopStats* out;
     int spc;           // sites per CTA (set by the launcher)
     int vs;            // 1: own basis rows kept in shared memory (set by the launcher)
     int lsw;           // 1: one extra warp runs the least-squares updates (set by the launcher)
     int ash;           // 1: the FP16 blocks of the first directions are kept in shared memory
                        // (set by the launcher)
+    int ks;            // FP64 push mode: column groups a row's apply is split over (set by the launcher)
     int dc;            // 1: delayed CGS2, one exchange per Arnoldi step (dataflow push mode)
     int flow;          // 1: push mode exchanges each step's values by st.async into byte-counted
                        // barriers instead of cluster barriers (set by the launcher)

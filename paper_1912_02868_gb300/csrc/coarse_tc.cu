@@ -17,9 +17,18 @@
 //  * Inner products.  A warp forms up to three products at once over half of the
 //    CTA's rows (PARTS = 2), so w is read once for all of them; the partials of
 //    both halves go into inbox rows of odd length (no bank conflicts).
-//  * The residual and the solution live in registers, the deflation space in
-//    shared memory when it fits; every exchange is dataflow, and the per-cycle
-//    cluster barrier (which only publishes faults) is split around the first one.
+//  * The residual and the solution live on chip, the deflation space too when it
+//    fits; every exchange is dataflow, and the per-cycle cluster barrier (which only
+//    publishes faults) is split around the first one.
+//
+// Grid form (GRID): coarse grids of more than one cluster's 256 sites run on one
+// cooperative grid over the whole GPU, a few sites a CTA.  An exchange then goes
+// through L2 without barrier or fence: every 4-byte value is stored with a 4-byte
+// tag of its exchange in one 8-byte word, and a reader polls the words themselves,
+// so a value costs one store and, once it is there, one load.  Two buffers by the
+// exchange's parity suffice: a CTA sends exchange e + 2 only after it has read e + 1,
+// which holds every CTA's contribution, made after that CTA had read e.  Each
+// projection exchange carries the CTAs' faults, so all leave together.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -40,6 +49,7 @@ namespace {
 // local memory misses the little L1 that the shared memory leaves).
 constexpr int SD = 2, SD1 = 4;
 constexpr int MAX_SITES = 16;
+constexpr int GRID_SPC = 8;  // grid form: sites a CTA, at least
 constexpr int XW = 48;      // words of one staged site: 12 entry pairs x (hi, hi, lo, lo)
 constexpr int OPA = SD * 3 * 32, OPB = SD1 * 3 * 32;  // fragments of one site in shared memory, by M tile
 
@@ -53,6 +63,10 @@ struct TcShape {
     int spc, halo, pw, ws, vrows;
     // byte offsets in dynamic shared memory
     int o_inbox, o_x, o_v, o_m, o_op, o_sol, o_w;
+    // GRID: tagged partial sums [2][PSTR][CTAs], tagged rows [2][sites x 24], and the tag
+    // base of this launch (advanced at its end)
+    ulonglong2 *part, *rows;
+    unsigned* epoch;
 };
 
 struct alignas(16) TcSmem {
@@ -78,6 +92,8 @@ struct alignas(16) TcSmem {
     int src[MAX_SITES][5];     // staged slot that holds the neighbour of each own site
     int hslot[MAX_SITES][4];   // slot of a neighbour owned by another CTA, -1 for an own site
     int nremote;
+    int hsite[MAX_SITES * 4];  // GRID: site of each neighbour slot
+    float anyf;                // GRID: faults of the projection exchange
 #ifdef CP_PHASE_CLOCKS
     int acc_t[16];
 #endif
@@ -109,14 +125,88 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
     return d;
 }
 
+__device__ __forceinline__ float4 both_orders(float2 v) { return make_float4(v.x, v.y, v.y, v.x); }
+
+// GRID: a tagged pair of words, and a polled read of N of them (those with bit i of
+// `have` clear are not read); false when the wait gave up
+__device__ __forceinline__ void st_tagged(ulonglong2* p, unsigned x, unsigned y, unsigned tag) {
+    const unsigned long long t = (unsigned long long)tag << 32;
+    asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};\n" ::"l"(p), "l"(t | x), "l"(t | y) : "memory");
+}
+__device__ __forceinline__ ulonglong2 ld_tagged(const ulonglong2* p) {
+    ulonglong2 v;
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];\n" : "=l"(v.x), "=l"(v.y) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ bool tagged(const ulonglong2& v, unsigned tag) {
+    return (unsigned)(v.x >> 32) == tag && (unsigned)(v.y >> 32) == tag;
+}
+
+// GRID: S.red / nrm as tc_reduce, from the CTAs' tagged partials gp[i][cta], i <= nd (and
+// the fault sum of product nd + 1 into *anyf where that is not null); false when a wait
+// gave up.  A warp takes values w and w + NW, all their partials (at most 160 CTAs) in
+// flight at once.
+constexpr int GRID_MAX = 160;
+template <int NW>
+__device__ __forceinline__ bool tc_reduce_grid(const ulonglong2* gp, int ncta, int nd, unsigned tag, long spin,
+                                               float4* red, float* nrm, float* anyf) {
+    constexpr int GP = GRID_MAX / 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int last = nd + (anyf ? 1 : 0), n4 = max((nd + 4) & ~3, last + 1);
+    bool ok = true;
+#pragma unroll 1
+    for (int i0 = warp; i0 < n4; i0 += 2 * NW) {
+        ulonglong2 q[2][GP];
+        unsigned wait = 0;  // bit h * GP + u: partial u of value i0 + h NW is still to come
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int u = 0; u < GP; ++u) {
+                q[h][u] = make_ulonglong2(0, 0);
+                if (i0 + h * NW <= last && lane + 32 * u < ncta) wait |= 1u << (h * GP + u);
+            }
+        for (long it = 0; wait && it < spin; ++it) {
+#pragma unroll
+            for (int b = 0; b < 2 * GP; ++b)
+                if ((wait >> b) & 1u) q[b / GP][b % GP] = ld_tagged(gp + (long)(i0 + b / GP * NW) * ncta + lane + 32 * (b % GP));
+#pragma unroll
+            for (int b = 0; b < 2 * GP; ++b)
+                if (((wait >> b) & 1u) && tagged(q[b / GP][b % GP], tag)) wait &= ~(1u << b);
+        }
+        ok = ok && wait == 0;
+        __syncwarp();
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int i = i0 + h * NW;
+            float2 v = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int u = 0; u < GP; ++u) {
+                v.x += __uint_as_float((unsigned)q[h][u].x);
+                v.y += __uint_as_float((unsigned)q[h][u].y);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+                v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+            }
+            if (lane == 0 && i < n4) {
+                if (i == nd) *nrm = v.x;
+                if (anyf && i == nd + 1) *anyf = v.x;
+                red[i] = i < nd ? both_orders(v) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+        }
+    }
+    return ok;
+}
+
 // Partial inner products conj(X[i]) . y, i < nd, and |y|^2 as product nd, over the
 // CTA's rows: a warp forms products 2w and 2w + 1 in one pass over y, two rows per
 // 16-byte load, and sends both in one 16-byte st.async to every CTA's inbox (row =
 // this CTA).  Packed FMAs: (Re Re, Im Im) and (Re Im, Im Re) of x and y are summed
 // as they lie; Re and Im of the product are their sum and difference.
-template <int NW>
+template <int NW, bool GRID>
 __device__ __forceinline__ void tc_gram(const float2* X, long ldx, int nd, const float2* y, int npairs, unsigned inbox,
-                                        int pw, unsigned bar, int nr, int me) {
+                                        int pw, unsigned bar, int nr, int me, ulonglong2* gp, unsigned tag) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const float4* y4 = reinterpret_cast<const float4*>(y);
 #pragma unroll 1
@@ -152,6 +242,12 @@ __device__ __forceinline__ void tc_gram(const float2* X, long ldx, int nd, const
             v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
             v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
         }
+        if constexpr (GRID) {
+            const int i = i0 + (lane >> 4);
+            if ((lane & 15) == 0 && i <= nd)
+                st_tagged(gp + (long)i * nr + me, __float_as_uint(v.x), __float_as_uint(v.y), tag);
+            continue;
+        }
         const float ox = __shfl_xor_sync(0xffffffffu, v.x, 16), oy = __shfl_xor_sync(0xffffffffu, v.y, 16);
         if (lane < nr)
             st_async4(cluster_addr(inbox + (unsigned)(me * pw + i0) * 8u, lane), __float_as_uint(v.x),
@@ -177,7 +273,6 @@ __device__ __forceinline__ double2 sqrt_rsqrt_d(float x) {
     return make_double2((double)x * y, y);
 }
 
-__device__ __forceinline__ float4 both_orders(float2 v) { return make_float4(v.x, v.y, v.y, v.x); }
 
 // red[i] = sum over the inbox rows of column i, i < nd (and column nd into *nrm), half
 // a warp a column, in one fixed tree (at most 16 rows): every CTA gets the same bits.
@@ -242,7 +337,7 @@ __device__ unsigned tc_clock_launches = 0;
 
 // NW warps.  NW = 8 serves at most 8 sites a CTA at two CTAs per SM, NW = 16 at most
 // 16 (128 registers a thread either way).
-template <int NW>
+template <int NW, bool GRID>
 __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1) k_coarse_tc(const __grid_constant__ CoopArgs<float> a,
                                                                         const __grid_constant__ TcShape g) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -263,6 +358,8 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1) k_coarse_tc(const __
     const int k = a.k, ms = a.ms;
     const int LD = MSMAX + 1;
 
+    const unsigned base = GRID ? __ldcg(g.epoch) : 0u;
+    unsigned ex = 0u, sx = 0u;  // GRID: exchanges and staged rows so far
     unsigned phases = 0u;  // parity of the next phase of barriers 0, 1, 2 (bits)
     // A wait that gives up marks the CTA faulted.  From then on the CTA skips its waits
     // and stops arming its barriers, and at the next round's cluster barrier every CTA
@@ -270,20 +367,22 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1) k_coarse_tc(const __
     // Only the last warp polls, the others wait at the CTA barrier that follows: polling
     // warps share the pipes of the shared-memory loads and shuffles of those still at work.
     auto flow_wait = [&](int b) {
-        if (warp != NW - 1) return;
+        if (GRID || warp != NW - 1) return;
         const unsigned par = (phases >> b) & 1u;
         phases ^= 1u << b;
         if (mbar_wait(&S.mb[b], par, 1)) return;
         if (!S.fault && !mbar_wait(&S.mb[b], par, a.spin > 0 ? a.spin : FLOW_SPIN)) S.fault = 1;
     };
     auto arm = [&](int b, int bytes) {
-        if (tid == NT - 32 && !S.fault) mbar_arm(&S.mb[b], (unsigned)bytes);
+        if (!GRID && tid == NT - 32 && !S.fault) mbar_arm(&S.mb[b], (unsigned)bytes);
     };
 
     // neighbour and push tables
     if (tid == 0) {
-        for (int b = 0; b < 4; ++b) mbar_init(&S.mb[b], 1);
-        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+        if (!GRID) {
+            for (int b = 0; b < 4; ++b) mbar_init(&S.mb[b], 1);
+            asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+        }
         S.fault = 0;
         int nrem = 0;
         for (int w = 0; w < my_sites; ++w) {
@@ -293,6 +392,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1) k_coarse_tc(const __
                 const bool own = u / g.spc == me;
                 S.hslot[w][d - 1] = own ? -1 : g.spc + nrem;
                 S.src[w][d] = own ? u - s0 : g.spc + nrem;
+                if (!own) S.hsite[nrem] = u;
                 nrem += own ? 0 : 1;
             }
         }
@@ -304,9 +404,16 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1) k_coarse_tc(const __
 #endif
     }
     for (int e = tid; e < 2 * MAX_CLUSTER; e += NT) (&S.fin[0][0])[e] = 0;
-    cluster_arrive();
-    cluster_wait();
-    if (tid < my_sites * 4) {
+    if (!GRID) {
+        cluster_arrive();
+        cluster_wait();
+    } else if (tid < my_sites) {  // own sites that another CTA reads (neighbours are mutual)
+        int out = -1;
+        for (int d = 1; d < 5; ++d)
+            if ((int)nbr_site(s0 + tid, d, a.Nx, a.Nt) / g.spc != me) out = 0;
+        S.push[tid][0] = out;
+    }
+    if (!GRID && tid < my_sites * 4) {
         const int w = tid >> 2, q = (tid & 3) + 1;
         const int from[5] = {0, 2, 1, 4, 3};  // dst = nbr(u, from[q]) reads u in direction q
         const int dst = (int)nbr_site(s0 + w, from[q], a.Nx, a.Nt), owner = dst / g.spc;
@@ -373,7 +480,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1) k_coarse_tc(const __
         V[tid] = a.f[(long)s0 * NDOF + tid];
     }
     __syncthreads();
-    if (a.probe && !S.fault && !mbar_wait(&S.mb[3], 0u, a.spin > 0 ? a.spin : FLOW_SPIN)) S.fault = 1;
+    if (!GRID && a.probe && !S.fault && !mbar_wait(&S.mb[3], 0u, a.spin > 0 ? a.spin : FLOW_SPIN)) S.fault = 1;
     // a new basis row: an even row stages itself and its odd partner, in the own
     // site's slot and in those of the neighbouring CTAs that read it
     auto stage = [&](float2 v) {
@@ -386,6 +493,14 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1) k_coarse_tc(const __
         if (row_on && !(lane & 1)) {
             const int site = tid / NDOF, off = (tid - site * NDOF) * 2;
             *reinterpret_cast<uint4*>(Xs + site * XW + off) = make_uint4(hi, hi1, lo, lo1);
+            if constexpr (GRID) {
+                if (S.push[site][0] >= 0) {
+                    ulonglong2* dst = g.rows + ((long)(sx & 1u) * nsite + s0) * NDOF + tid;
+                    st_tagged(dst, hi, lo, base + sx + 1u);
+                    st_tagged(dst + 1, hi1, lo1, base + sx + 1u);
+                }
+                return;
+            }
             const int4 p = *reinterpret_cast<const int4*>(S.push[site]);
             auto send = [&](int code) {
                 if (code < 0) return;
@@ -407,16 +522,47 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1) k_coarse_tc(const __
     // one exchange of nd inner products of X with y into S.red[buf], and |y|^2.  The
     // buffers alternate: a CTA sends into buffer b only after an exchange on the other
     // one, to which this CTA contributes after it has read buffer b.
-    auto exchange = [&](int buf, const float2* X, long ldx, int nd, const float2* y) {
+    auto exchange = [&](int buf, const float2* X, long ldx, int nd, const float2* y, bool faults = false) {
         arm(buf, ncta * ((nd + 2) & ~1) * 8);
         const unsigned in = smem_addr(inbox0) + (unsigned)(buf * MAX_CLUSTER * g.pw) * 8u;
-        tc_gram<NW>(X, ldx, nd, y, nrows >> 1, in, g.pw, smem_addr(&S.mb[buf]), ncta, me);
+        ulonglong2* gp = GRID ? g.part + (long)(ex & 1u) * PSTR * ncta : nullptr;
+        tc_gram<NW, GRID>(X, ldx, nd, y, nrows >> 1, in, g.pw, smem_addr(&S.mb[buf]), ncta, me, gp, base + ex + 1u);
         TC_STAMP(8);
-        flow_wait(buf);
+        if constexpr (GRID) {
+            if (faults && tid == NT - 1)
+                st_tagged(gp + (long)(nd + 1) * ncta + me, __float_as_uint(S.fault ? 1.f : 0.f), 0u, base + ex + 1u);
+            const long spin = S.fault ? 0 : (a.spin > 0 ? a.spin : FLOW_SPIN);
+            if (!tc_reduce_grid<NW>(gp, ncta, nd, base + ex + 1u, spin, S.red[buf], &S.nrm[buf],
+                                    faults ? &S.anyf : nullptr))
+                S.fault = 1;
+            ++ex;
+        } else {
+            flow_wait(buf);
+            __syncthreads();
+            TC_STAMP(9);
+            tc_reduce<NW>(inbox0 + buf * MAX_CLUSTER * g.pw, ncta, g.pw, nd, S.red[buf], &S.nrm[buf]);
+        }
         __syncthreads();
-        TC_STAMP(9);
-        tc_reduce<NW>(inbox0 + buf * MAX_CLUSTER * g.pw, ncta, g.pw, nd, S.red[buf], &S.nrm[buf]);
-        __syncthreads();
+    };
+    // GRID: the neighbouring CTAs' rows of the staged vector into their slots
+    auto receive = [&]() {
+        if constexpr (GRID) {
+            const ulonglong2* src = g.rows + (long)(sx & 1u) * nsite * NDOF;
+            for (int e = tid; e < S.nremote * (NDOF / 2); e += NT) {
+                const int slot = e / (NDOF / 2), m = e - slot * (NDOF / 2);
+                const ulonglong2* p = src + (long)S.hsite[slot] * NDOF + 2 * m;
+                ulonglong2 q0, q1;
+                long it = S.fault ? 0 : (a.spin > 0 ? a.spin : FLOW_SPIN);
+                do {
+                    q0 = ld_tagged(p);
+                    q1 = ld_tagged(p + 1);
+                } while (!(tagged(q0, base + sx + 1u) && tagged(q1, base + sx + 1u)) && --it > 0);
+                if (it <= 0) S.fault = 1;
+                *reinterpret_cast<uint4*>(Xs + (g.spc + slot) * XW + m * 4) =
+                    make_uint4((unsigned)q0.x, (unsigned)q1.x, (unsigned)q0.y, (unsigned)q1.y);
+            }
+            ++sx;
+        }
     };
     int cycles = 0;
     // Least squares of the cycle, by the last warp while the staged rows travel.  The
@@ -467,18 +613,22 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1) k_coarse_tc(const __
         // ---- projection onto the deflation space: d = argmin ||W^+ r - H_k d|| ----
         // Every CTA publishes its fault to all before the split cluster barrier; all
         // read the same flags after it, the one place where CTAs leave.
-        if (warp == 0 && lane < ncta) {
-            const unsigned ra = cluster_addr(smem_addr(&S.fin[cycles & 1][me]), lane);
-            asm volatile("st.shared::cluster.b32 [%0], %1;\n" ::"r"(ra), "r"(S.fault) : "memory");
+        if (!GRID) {
+            if (warp == 0 && lane < ncta) {
+                const unsigned ra = cluster_addr(smem_addr(&S.fin[cycles & 1][me]), lane);
+                asm volatile("st.shared::cluster.b32 [%0], %1;\n" ::"r"(ra), "r"(S.fault) : "memory");
+            }
+            __syncwarp();
+            cluster_arrive();
         }
-        __syncwarp();
-        cluster_arrive();
         const float2* Wl = g.ws ? reinterpret_cast<const float2*>(smem_raw + g.o_w) : a.W + (long)s0 * NDOF;
         const long ldw = g.ws ? ldv : (long)nsite * NDOF;
-        exchange(0, Wl, ldw, k + 1, V);
-        cluster_wait();
+        exchange(0, Wl, ldw, k + 1, V, true);
+        if (!GRID) cluster_wait();
         int anyf = 0;
-        for (int q = 0; q < ncta; ++q) anyf |= S.fin[cycles & 1][q];
+        if (GRID) anyf = S.fault | (S.anyf != 0.f);
+        else
+            for (int q = 0; q < ncta; ++q) anyf |= S.fin[cycles & 1][q];
         // S.ctl[0]: the last cycle converged (the same in every CTA that has not faulted)
         if (anyf | S.ctl[0] | (cycles >= a.max_cycles)) break;
         if (cycles == 0 && tid == 0)  // r = f: the tolerance is relative to ||f||
@@ -540,6 +690,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1) k_coarse_tc(const __
         for (; j < ms; ++j) {
             float2* const wl = V + (j + 1) * ldv;
             flow_wait(2);     // v_j staged by the neighbouring CTAs
+            receive();
             __syncthreads();  // and by the own warps
             TC_STAMP(0);
             if (site_warp) {  // w = A v_j at site `warp`
@@ -634,6 +785,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1) k_coarse_tc(const __
         }
         if (j == ms) {     // the last step's update, when no stop came before
             flow_wait(2);  // the staging of v_ms, which no apply reads
+            ++sx;
             __syncthreads();
         }
         if (tid == 0) S.iters += j;
@@ -698,12 +850,17 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1) k_coarse_tc(const __
                S.acc_t[5] / clk_steps, S.acc_t[12] / clk_steps, S.acc_t[13] / clk_steps, S.acc_t[6] / clk_steps,
                S.acc_t[7] / clk_steps);
 #endif
-    cluster_arrive();  // no CTA leaves while others may still write its shared memory
-    cluster_wait();
+    if (GRID) {
+        // (every CTA has read the base: this one has had a whole exchange from all of them)
+        if (me == 0 && tid == 0) *g.epoch = base + max(ex, sx) + 1u;
+    } else {
+        cluster_arrive();  // no CTA leaves while others may still write its shared memory
+        cluster_wait();
+    }
 }
 
 struct TcGeometry {
-    int ok = 0, ctas = 0, nw = 0;
+    int ok = 0, ctas = 0, nw = 0, grid = 0;
     size_t smem = 0;
     TcShape g{};
 };
@@ -729,9 +886,9 @@ int max_halo(int Nx, int Nt, int spc) {
 }
 
 template <int NW>
-bool fits(TcGeometry& G, bool set_attr) {
-    auto* kern = k_coarse_tc<NW>;
-    if (set_attr) {
+bool fits(TcGeometry& G) {
+    auto* kern = k_coarse_tc<NW, false>;
+    {
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_LIMIT) != cudaSuccess ||
             cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
             (void)cudaGetLastError();
@@ -756,52 +913,76 @@ bool fits(TcGeometry& G, bool set_attr) {
     return nc >= 1;
 }
 
+// shared-memory layout for spc sites a CTA; two: leave room for two CTAs per SM when
+// that costs only the deflation space's copy
+void tc_layout(int Nx, int Nt, int ms, int k, int spc, bool two, TcGeometry& G) {
+    TcShape& g = G.g;
+    g = TcShape{};
+    g.spc = spc;
+    G.ctas = (Nx * Nt + spc - 1) / spc;
+    // an inbox row holds its products and the norm, in 16-byte pairs; rows an odd
+    // number of pairs apart fall on different banks
+    g.pw = (std::max(k + 2, ms + 1) + 1) & ~1;
+    if (g.pw % 4 == 0) g.pw += 2;
+    g.halo = max_halo(Nx, Nt, spc);
+    size_t o = (sizeof(TcSmem) + 15) & ~size_t(15);
+    auto take = [&](size_t bytes) {
+        const size_t at = o;
+        o = (o + bytes + 15) & ~size_t(15);
+        return (int)at;
+    };
+    const size_t rows = (size_t)spc * NDOF;
+    g.o_inbox = take(G.grid ? 0 : (size_t)2 * MAX_CLUSTER * g.pw * sizeof(float2));
+    g.o_x = take(std::max((size_t)(spc + g.halo) * XW * 4, (size_t)(MSMAX + 1) * MSMAX * sizeof(float2)));
+    g.vrows = std::max(ms + 1, (ms + 3) & ~3);  // row updates read whole groups of four rows
+    g.o_v = take((size_t)g.vrows * rows * sizeof(float2));
+    g.o_sol = take(rows * sizeof(float2));
+    g.o_m = take((size_t)(2 * k + 1) * (k + 1) * sizeof(float2));
+    g.o_op = take((size_t)spc * (OPA * 16 + OPB * 8));
+    const size_t base = o, with_w = o + (size_t)(k + 1) * rows * sizeof(float2);
+    const size_t half = (SMEM_LIMIT - 1024) / 2;
+    g.ws = (with_w <= half || (with_w <= SMEM_LIMIT && (!two || base > half))) ? 1 : 0;
+    g.o_w = (int)base;
+    G.smem = g.ws ? with_w : base;
+}
+
 void tc_geometry_uncached(int Nx, int Nt, int ms, int k, TcGeometry& G) {
     const int nsite = Nx * Nt;
-    for (int cl = MAX_CLUSTER; cl >= 1; cl >>= 1) {
-        const int spc = (nsite + cl - 1) / cl;
-        if (spc > MAX_SITES) return;
-        TcShape& g = G.g;
-        g = TcShape{};
-        g.spc = spc;
-        G.ctas = (nsite + spc - 1) / spc;
-        G.nw = spc <= 8 ? 8 : 16;
-        // an inbox row holds its products and the norm, in 16-byte pairs; rows an odd
-        // number of pairs apart fall on different banks
-        g.pw = (std::max(k + 2, ms + 1) + 1) & ~1;
-        if (g.pw % 4 == 0) g.pw += 2;
-        g.halo = max_halo(Nx, Nt, spc);
-        size_t o = (sizeof(TcSmem) + 15) & ~size_t(15);
-        auto take = [&](size_t bytes) {
-            const size_t at = o;
-            o = (o + bytes + 15) & ~size_t(15);
-            return (int)at;
-        };
-        const size_t rows = (size_t)spc * NDOF;
-        g.o_inbox = take((size_t)2 * MAX_CLUSTER * g.pw * sizeof(float2));
-        g.o_x = take(std::max((size_t)(spc + g.halo) * XW * 4, (size_t)(MSMAX + 1) * MSMAX * sizeof(float2)));
-        g.vrows = std::max(ms + 1, (ms + 3) & ~3);  // row updates read whole groups of four rows
-        g.o_v = take((size_t)g.vrows * rows * sizeof(float2));
-        g.o_sol = take(rows * sizeof(float2));
-        g.o_m = take((size_t)(2 * k + 1) * (k + 1) * sizeof(float2));
-        g.o_op = take((size_t)spc * (OPA * 16 + OPB * 8));
-        const size_t base = o, with_w = ((o + (size_t)(k + 1) * rows * sizeof(float2)) + 15) & ~size_t(15);
-        const size_t half = (SMEM_LIMIT - 1024) / 2;  // two CTAs per SM
-        // the deflation space in shared memory where that costs no resident CTA
-        g.ws = (with_w <= half || (with_w <= SMEM_LIMIT && (G.nw == 16 || base > half))) ? 1 : 0;
-        g.o_w = (int)base;
-        G.smem = g.ws ? with_w : base;
-        if (G.smem > SMEM_LIMIT) continue;
-        G.ok = (G.nw == 8 ? fits<8>(G, true) : fits<16>(G, true)) ? 1 : 0;
-        if (G.ok) return;
+    if (nsite <= MAX_CLUSTER * MAX_SITES) {
+        for (int cl = MAX_CLUSTER; cl >= 1; cl >>= 1) {
+            const int spc = (nsite + cl - 1) / cl;
+            if (spc > MAX_SITES) return;
+            G.nw = spc <= 8 ? 8 : 16;
+            tc_layout(Nx, Nt, ms, k, spc, G.nw == 8, G);
+            if (G.smem > SMEM_LIMIT) continue;
+            G.ok = (G.nw == 8 ? fits<8>(G) : fits<16>(G)) ? 1 : 0;
+            if (G.ok) return;
+        }
+        return;
     }
+    // grid form: the fewest CTAs that keep a CTA's step short, one per SM
+    G.nw = 16;
+    G.grid = 1;
+    const int most = std::min(sm_count(), GRID_MAX);
+    const int spc = std::max(GRID_SPC, (nsite + most - 1) / most);
+    if (spc > MAX_SITES) return;
+    tc_layout(Nx, Nt, ms, k, spc, false, G);
+    if (G.smem > SMEM_LIMIT) return;
+    int per_sm = 0;
+    if (cudaFuncSetAttribute(k_coarse_tc<16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_LIMIT) !=
+            cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_coarse_tc<16, true>, 512, G.smem) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return;
+    }
+    G.ok = per_sm >= 1 && G.ctas <= per_sm * sm_count() ? 1 : 0;
 }
 
 }  // namespace
 
 mg_status launch_coarse_tc(const CoopArgs<float>& a, cudaStream_t s, bool* launched) {
     *launched = false;
-    if (!a.Ah || !a.mma || a.dc || (long)a.Nx * a.Nt > (long)MAX_CLUSTER * MAX_SITES) return MG_OK;
+    if (!a.Ah || !a.mma || a.dc || (long)a.Nx * a.Nt > (long)GRID_MAX * MAX_SITES) return MG_OK;
     struct Entry {
         int dev, Nx, Nt, ms, k;
         TcGeometry G;
@@ -825,20 +1006,29 @@ mg_status launch_coarse_tc(const CoopArgs<float>& a, cudaStream_t s, bool* launc
             cache.push_back(Entry{dev, a.Nx, a.Nt, a.ms, a.k, G});
         }
     }
-    if (!G.ok) return MG_OK;
+    if (!G.ok || (G.grid && (!a.part || !a.rows))) return MG_OK;
+    G.g.part = reinterpret_cast<ulonglong2*>(a.part);
+    G.g.rows = reinterpret_cast<ulonglong2*>(a.rows);
+    G.g.epoch = a.epoch;
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = G.ctas;
-    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    if (G.grid) {
+        attr[0].id = cudaLaunchAttributeCooperative;
+        attr[0].val.cooperative = 1;
+    } else {
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = G.ctas;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    }
     cfg.gridDim = dim3(G.ctas);
     cfg.blockDim = dim3(G.nw * 32);
     cfg.dynamicSmemBytes = G.smem;
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (G.nw == 8) MG_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_coarse_tc<8>, a, G.g));
-    else MG_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_coarse_tc<16>, a, G.g));
+    if (G.grid) MG_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_coarse_tc<16, true>, a, G.g));
+    else if (G.nw == 8) MG_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_coarse_tc<8, false>, a, G.g));
+    else MG_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_coarse_tc<16, false>, a, G.g));
     count_launch();
     *launched = true;
     return MG_OK;

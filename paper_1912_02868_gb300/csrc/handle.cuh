@@ -153,8 +153,12 @@ struct Handle {
     DRState* dr = nullptr;
     KState* pls = nullptr;    // factored H_k of the deflation space
     ProjMats* pmat = nullptr; // its projection matrices
-    double2* cpart = nullptr; // partial sums of the cooperative coarse solve
+    // exchange buffers of the coarse solve over the whole GPU (grids of more than one
+    // cluster's sites): tagged partial sums, tagged rows, tag base
+    double2* cpart = nullptr;
     int cpart_ctas = 0;
+    double2* crows = nullptr;
+    unsigned* cepoch = nullptr;
     CoopStats* cstats = nullptr;
     // fine-grid deflation arm (method MG_METHOD_FINE_DEFLATION), FP64
     double2* fdV = nullptr;   // (m+1) x n0
@@ -195,6 +199,9 @@ template <> inline PartialWS<float>& Handle::partial<float>() { return p32; }
 
 // allocation owned by the handle
 mg_status halloc(Handle& H, void** p, size_t bytes);
+// clears the exchange buffers of the grid-wide coarse solve (at allocation, and after a
+// solve in which a wait gave up: its CTAs' tags may have run apart)
+mg_status clear_coarse_exchange(Handle& H, cudaStream_t s);
 template <typename P> mg_status halloc_t(Handle& H, P** p, size_t count) {
     return halloc(H, reinterpret_cast<void**>(p), count * sizeof(P));
 }

@@ -306,6 +306,8 @@ CoopArgs<T> proj_args(Handle& H, const C2<T>* f, C2<T>* x) {
     a.max_cycles = H.p.proj_max_cycles;
     a.part = H.cpart;
     a.part_ctas = H.cpart_ctas;
+    a.rows = H.crows;
+    a.epoch = H.cepoch;
     a.out = H.cstats;
     a.Ah = std::is_same<T, float>::value ? H.A16c : nullptr;
     a.dc = H.p.coarse_dcgs2;
