@@ -55,6 +55,7 @@ using namespace cdev;
 namespace {
 
 constexpr int MAX_THREADS = 512;
+constexpr int F64_ROW_THREADS = 480;  // row threads of the FP64 push mode (with the least-squares warp: 512)
 constexpr int MAX_SPC = 16;       // sites per apply chunk (staged neighbour rows)
 constexpr int MAX_NB_SITES = 64;  // sites per CTA in the neighbour table
 // FP16 operator (push mode): the blocks of directions 0..ASH_DIRS-1 of a CTA's
@@ -124,6 +125,39 @@ __device__ __forceinline__ void st_rank(C2<T>* dst, int rank, int me, C2<T> v) {
         asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};\n" ::"r"(ra), "f"(v.x), "f"(v.y) : "memory");
     else
         asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};\n" ::"r"(ra), "d"(v.x), "d"(v.y) : "memory");
+}
+
+// FP64 forms of the inner products and reductions below.  An FP64 instruction of a
+// warp takes 64 cycles of its scheduler however many lanes are active, so the forms
+// here spend as few of them as they can: two products share a warp's butterfly, each
+// half warp keeping one and then each quarter one part of it (6 additions for two
+// complex sums instead of 20).
+//
+// After it, lanes 0, 8, 16 and 24 hold a.x, a.y, b.x and b.y summed over the warp;
+// every lane returns both sums.
+__device__ __forceinline__ void warp_sum_pair(double2& a, double2& b) {
+    const int lane = threadIdx.x & 31;
+    const bool hi = lane & 16, im = lane & 8;
+    double2 v = hi ? b : a;
+    v.x += __shfl_xor_sync(0xffffffffu, hi ? a.x : b.x, 16);
+    v.y += __shfl_xor_sync(0xffffffffu, hi ? a.y : b.y, 16);
+    double w = (im ? v.y : v.x) + __shfl_xor_sync(0xffffffffu, im ? v.x : v.y, 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+    a.x = __shfl_sync(0xffffffffu, w, 0);
+    a.y = __shfl_sync(0xffffffffu, w, 8);
+    b.x = __shfl_sync(0xffffffffu, w, 16);
+    b.y = __shfl_sync(0xffffffffu, w, 24);
+}
+// conj(X[i]) . y and conj(X[i + 1]) . y over this lane's rows, two chains each
+__device__ __forceinline__ void lane_products(const double2* xa, const double2* xb, const double2* y, int nrows,
+                                              double2& a, double2& b) {
+    a = b = make_double2(0.0, 0.0);
+    for (int e = threadIdx.x & 31; e < nrows; e += 32) {
+        const double2 ye = y[e];
+        a = cfmac(xa[e], ye, a);
+        b = cfmac(xb[e], ye, b);
+    }
 }
 
 // Partials of nd inner products conj(X[i]) . y over the CTA's rows (X, y point
@@ -219,6 +253,25 @@ __device__ __forceinline__ void accum_rows2(C2<T>& acc0, C2<T>& acc1, const C2<T
 template <typename T>
 __device__ void reduce_inbox(const C2<T>* inbox, int nr, int n, C2<T>* red, int nw) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if constexpr (std::is_same<T, double>::value) {
+        // half a warp a value, its halves one part each: 4 additions for two values
+        const int l = lane & 15;
+        const bool im = lane & 8;
+        for (int i0 = 2 * warp; i0 < n && warp < nw; i0 += 2 * nw) {
+            const int i = i0 + (lane >> 4);
+            C2<T> a = mk<T>(0, 0);
+            if (l < nr && i < n) a = inbox[l * PSTR + i];
+            T w = (im ? a.y : a.x) + __shfl_xor_sync(0xffffffffu, im ? a.x : a.y, 8);
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+            if ((lane & 7) == 0 && i < n) {
+                if (im) red[i].y = w;
+                else red[i].x = w;
+            }
+        }
+        __syncthreads();
+        return;
+    }
     for (int i = warp; i < n && warp < nw; i += nw) {
         C2<T> a = mk<T>(0, 0);
         if (lane < nr) a = inbox[lane * PSTR + i];
@@ -254,6 +307,20 @@ __device__ void push_gram_flow(const C2<T>* X, long ldx, int nd, const C2<T>* y,
     if (warp >= nw) return;
     const int ntot = nd + (norm ? 1 : 0);
     const unsigned bar_r = lane < nr ? cluster_addr(smem_addr(bar), lane) : 0u;
+    if constexpr (std::is_same<T, double>::value) {
+        for (int i = 2 * warp; i < ntot; i += 2 * nw) {
+            C2<T> p, q;
+            lane_products(i < nd ? X + (long)i * ldx : y, i + 1 < nd ? X + (long)(i + 1) * ldx : y, y, nrows, p, q);
+            warp_sum_pair(p, q);
+            if (i >= nd) p.y = 0;
+            if (i + 1 >= nd) q.y = 0;
+            if (lane < nr) {
+                st_async(cluster_addr(smem_addr(inbox + me * PSTR + i), lane), p, bar_r);
+                if (i + 1 < ntot) st_async(cluster_addr(smem_addr(inbox + me * PSTR + i + 1), lane), q, bar_r);
+            }
+        }
+        return;
+    }
     for (int i = warp; i < ntot; i += nw) {
         C2<T> acc4[4];
 #pragma unroll
@@ -416,6 +483,8 @@ __global__ void __maxnreg__(128) k_coarse_proj(CoopArgs<T> a) {
     for (int e = tid; e < k * (k + 1); e += nt) Mp[e] = from_d2<T>(a.pm->M[e]);
     for (int e = tid; e < (k + 1) * (k + 1); e += nt) Np[e] = from_d2<T>(a.pm->N[e]);
 
+    // FP64 apply split over column groups (a.ks > 1): partial sums [ks][rows]
+    Z* Psum = Np + (k + 1) * (k + 1);
     // a.ash: the FP16 blocks of the first ASH_DIRS directions of the own sites,
     // copied once into shared memory after M and N
     unsigned* Ash = reinterpret_cast<unsigned*>(Np + (k + 1) * (k + 1));
@@ -447,7 +516,45 @@ __global__ void __maxnreg__(128) k_coarse_proj(CoopArgs<T> a) {
     // (h1 + h2, h_{jc+1,jc}), the previous rotations applied to it, the new
     // rotation, and the stop flags from the residual estimate |g_{jc+1}|.  Reads
     // S.h1 and S.red, which the step after jc overwrites only after its apply.
+    Z u_ls = mk<T>(0, 0), g_ls = mk<T>(0, 0);
     auto ls_update = [&](int lane, int jc, T hnv) {
+        if constexpr (std::is_same<T, double>::value) {
+            // The rotations turn column j's running entry into p_{t+1} = c_t h_{t+1} -
+            // conj(s_t) p_t, so the entry that meets h_{j+1,j} is a dot product p = sum u_i h_i
+            // with u^{(j+1)} = (-conj(s_j) u^{(j)}, c_j): lane i keeps u_i, and a step costs one
+            // warp sum instead of a chain of j rotations at this GPU's FP64 latency.  The rotated
+            // columns are formed at the cycle's end, one lane a column.
+            Z h = mk<T>(0, 0);
+            if (lane <= jc) {
+                h = cadd(S.h1[lane], S.red[lane]);
+                st.H[lane + LD * jc] = h;
+            } else if (lane == jc + 1) {
+                st.H[lane + LD * jc] = mk<T>(hnv, 0);
+            }
+            if (jc == 0) {
+                u_ls = mk<T>(lane == 0 ? T(1) : T(0), 0);
+                g_ls = st.c[0];
+            }
+            Z p = cmul(u_ls, h), z = mk<T>(0, 0);
+            warp_sum_pair(p, z);
+            T cc;
+            Z ss, rv;
+            givens_real_<T>(p, hnv, cc, ss, rv);
+            const Z msc = cneg(conj_(ss));
+            u_ls = lane == jc + 1 ? mk<T>(cc, 0) : cmul(msc, u_ls);
+            if (lane == 0) {
+                st.rc[jc] = cc;
+                st.rs[jc] = ss;
+                st.g[jc] = cscale(g_ls, cc);
+            }
+            g_ls = cmul(msc, g_ls);
+            if (lane == 0) {
+                S.ctl[0] = (g_ls.x * g_ls.x + g_ls.y * g_ls.y <= tol_abs * tol_abs) ? 1 : 0;
+                S.ctl[1] = (hnv == T(0)) ? 1 : 0;
+            }
+            __syncwarp();
+            return;
+        }
         for (int i = lane; i <= jc; i += 32) st.H[i + LD * jc] = cadd(S.h1[i], S.red[i]);
         if (lane == 0) st.H[(jc + 1) + LD * jc] = mk<T>(hnv, 0);
         __syncwarp();
@@ -662,6 +769,22 @@ __global__ void __maxnreg__(128) k_coarse_proj(CoopArgs<T> a) {
         conv = S.ctl[0];
         return ms;
     };
+    // Row updates w - V h of few rows in FP64 (one site a CTA): PS adjacent lanes share a
+    // row's products, so that three schedulers work instead of one
+    constexpr int PS = 4;
+    const bool split_rows = std::is_same<T, double>::value && flow && a.lsw && nrows * PS <= 96 && nwr * 32 >= 96;
+    auto accum_split = [&](const Z* w, const Z* h, int cnt) {
+        const int e = tid / PS, q0 = tid % PS;
+        Z acc = q0 == 0 ? w[e] : mk<T>(0, 0);
+        for (int i = q0; i < cnt; i += PS) acc = cfms_<T>(Vl[(long)i * ldv + e], h[i], acc);
+        const unsigned m = __activemask();
+#pragma unroll
+        for (int o = PS / 2; o > 0; o >>= 1) {
+            acc.x += __shfl_xor_sync(m, acc.x, o);
+            acc.y += __shfl_xor_sync(m, acc.y, o);
+        }
+        return acc;
+    };
     while (true) {
         // ---- projection onto the deflation space: d = argmin ||W^+ r - H_k d|| ----
         if (tid == 0) S.fpub[cycles & 1] = S.fault;
@@ -783,6 +906,31 @@ __global__ void __maxnreg__(128) k_coarse_proj(CoopArgs<T> a) {
                         }
                         wl[(long)c0 * NDOF + e] = acc;
                     }
+                } else if (std::is_same<T, double>::value && a.ks > 1) {
+                    // few rows in FP64: column group q of a row on its own thread (the groups fill
+                    // the warps, so the row's DFMAs spread over all four schedulers), then the
+                    // groups' partial sums
+                    const int cols = 5 * NDOF / a.ks;
+                    if (tid < nrows * a.ks) {
+                        const int q = tid / nrows, e = tid - q * nrows, ls = e / NDOF, kk = e - ls * NDOF;
+                        const Z* Ab = a.A + (s0 + ls) * (5L * NDOF * NDOF) + (long)q * cols * NDOF + kk;
+                        const Z* xq = &S.xs[ls][0][0] + q * cols;
+                        Z acc = mk<T>(0, 0);
+#pragma unroll 6
+                        for (int l = 0; l < cols; ++l) acc = cfma(__ldg(Ab + l * NDOF), xq[l], acc);
+                        Psum[tid] = acc;
+                    }
+                    if (!ls_warp) row_warps_sync(nwr * 32);
+                    // each real component by itself; with many groups, four lanes a component
+                    const T* ps = reinterpret_cast<const T*>(Psum);
+                    const int ql = a.ks >= 12 ? 4 : 1;
+                    if (tid < 2 * nrows * ql) {
+                        const int c = tid / ql, q0 = tid - c * ql;
+                        T acc = 0;
+                        for (int q = q0; q < a.ks; q += ql) acc += ps[(long)q * 2 * nrows + c];
+                        for (int o = ql >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(__activemask(), acc, o);
+                        if (q0 == 0) reinterpret_cast<T*>(wl)[c] = acc;
+                    }
                 } else {
                     for (int e = tid; e < cs * NDOF; e += nt) {
                         const int ls = e / NDOF, kk = e - ls * NDOF;
@@ -814,7 +962,14 @@ __global__ void __maxnreg__(128) k_coarse_proj(CoopArgs<T> a) {
             }
             CP_STAMP(2);
             reduce_inbox<T>(&S.inbox[1][0][0], ncta, j + 1, S.h1, nwr);
-            for (int e = tid; e < nrows; e += nt) wl[e] = accum_rows<T, true>(wl[e], Vl, ldv, e, S.h1, j + 1);
+            if (split_rows) {
+                if (tid < nrows * PS) {
+                    const Z v = accum_split(wl, S.h1, j + 1);
+                    if (tid % PS == 0) wl[tid / PS] = v;
+                }
+            } else {
+                for (int e = tid; e < nrows; e += nt) wl[e] = accum_rows<T, true>(wl[e], Vl, ldv, e, S.h1, j + 1);
+            }
             __syncthreads();
             CP_STAMP(3);
             if (flow) {
@@ -829,16 +984,41 @@ __global__ void __maxnreg__(128) k_coarse_proj(CoopArgs<T> a) {
             reduce_inbox<T>(&S.inbox[0][0][0], ncta, j + 2, S.red, nwr);
             // h_{j+1,j} = ||w - V h2|| = sqrt(n2 - |h2|^2) (V orthonormal), computed
             // identically by every thread; then v_{j+1} = (w - V h2) / h_{j+1,j}
-            T h2n = 0;  // warp butterfly: the same value in every lane and warp
-            for (int i = tid & 31; i <= j; i += 32) h2n += S.red[i].x * S.red[i].x + S.red[i].y * S.red[i].y;
+            T hn = 0, sc = 0;
+            // (in FP64 only by the warps that use it: every warp's sums take the FP64 pipe)
+            if (!std::is_same<T, double>::value || ls_warp || !a.lsw || (tid & ~31) < nrows * (split_rows ? PS : 1)) {
+                T h2n = 0;  // warp butterfly: the same value in every lane and warp
+                for (int i = tid & 31; i <= j; i += 32) h2n += S.red[i].x * S.red[i].x + S.red[i].y * S.red[i].y;
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) h2n += __shfl_xor_sync(0xffffffffu, h2n, o);
-            const T hn = sqrt(fmax((T)S.red[j + 1].x - h2n, T(0)));
+                for (int o = 16; o > 0; o >>= 1) h2n += __shfl_xor_sync(0xffffffffu, h2n, o);
+                const T hh = fmax((T)S.red[j + 1].x - h2n, T(0));
+                if constexpr (std::is_same<T, double>::value) {
+                    // one reciprocal square root and a correction step instead of the square
+                    // root and the division one after the other
+                    if (hh > T(0)) {
+                        sc = rsqrt(hh);
+                        hn = hh * sc;
+                        hn = fma(fma(-hn, hn, hh), T(0.5) * sc, hn);
+                    }
+                } else {
+                    hn = sqrt(hh);
+                    sc = hn > T(0) ? T(1) / hn : T(0);
+                }
+            }
             {
-                const T sc = hn > T(0) ? T(1) / hn : T(0);
                 Z* wg = a.V + (long)(j + 1) * n + r0;
                 if (flow) arm(2, (unsigned)(my_sites * 5 * NDOF * sizeof(Z)));
-                for (int e = tid; e < nrows; e += nt) {
+                if (split_rows && tid < nrows * PS) {  // dataflow mode: the lanes of a row share its pushes
+                    const int e = tid / PS, q0 = tid % PS, ls = e / NDOF, kk = e - ls * NDOF;
+                    const Z v = cscale(accum_split(wl, S.red, j + 1), sc);
+                    if (q0 == 0) wl[e] = v;
+                    for (int q = q0; q < 5; q += PS) {
+                        const int code = S.pusht[ls][q], owner = code >> 16;
+                        st_async(cluster_addr(smem_addr(&S.xs[(code >> 3) & 0x1fff][code & 7][kk]), owner), v,
+                                 cluster_addr(smem_addr(&S.mb[2]), owner));
+                    }
+                }
+                for (int e = tid; e < nrows && !split_rows; e += nt) {
                     const Z v = cscale(accum_rows<T, true>(wl[e], Vl, ldv, e, S.red, j + 1), sc);
                     wl[e] = v;
                     if (flow)
@@ -886,7 +1066,19 @@ __global__ void __maxnreg__(128) k_coarse_proj(CoopArgs<T> a) {
         }
         // ---- finish the cycle: d = R^{-1} g, rho = c - H d, x += V d, r = V rho ----
         const int jj = j;
-        if (tid < 32) back_subst_warp<T>(st.Rm, st.g, st.d, jj, tid);
+        if (tid < 32) {
+            if (std::is_same<T, double>::value && !dc && tid < jj) {  // column tid of R (see ls_update)
+                Z p = st.H[LD * tid];
+                for (int t = 0; t <= tid; ++t) {
+                    Z q = st.H[LD * tid + t + 1];
+                    rot_<T>(st.rc[t], st.rs[t], p, q);
+                    st.Rm[t + LD * tid] = p;
+                    p = q;
+                }
+            }
+            __syncwarp();
+            back_subst_warp<T>(st.Rm, st.g, st.d, jj, tid);
+        }
         __syncthreads();
         for (int i = tid; i <= jj; i += nt) {
             Z acc = st.c[i];
@@ -1415,7 +1607,7 @@ __global__ void __maxnreg__(128) k_coarse_proj_pair(CoopArgs<T> a0, CoopArgs<T> 
 }
 
 struct Geometry {
-    int cluster = 1, spc = 1, threads = 32, vs = 0, lsw = 0, ash = 0;
+    int cluster = 1, spc = 1, threads = 32, vs = 0, lsw = 0, ash = 0, ks = 1;
     size_t smem = 0, smem_ash = 0;  // dynamic shared memory without / with the shared FP16 blocks
 };
 
@@ -1438,12 +1630,20 @@ mg_status geometry_uncached(long nsite, int ms, int k, int dev, Geometry& g) {
         int threads = ((rows + 31) / 32) * 32;
         threads = std::min(std::max(threads, 64), MAX_THREADS);
         for (int vs = 1; vs >= 0; --vs) {
-            const size_t smem = sizeof(ClusterSmem<T>) + (vs ? slice_bytes<T>(ms, rows) : 0) + proj_bytes<T>(k);
-            if (smem > SMEM_LIMIT) continue;
             // push mode (basis in shared memory, one staging chunk) gets the extra
             // least-squares warp
             const int lsw = (vs && spc <= MAX_SPC) ? 1 : 0;
-            const int thr = threads + 32 * lsw;
+            // FP64 push mode: 480 row threads however few the rows, the apply split over
+            // the largest number of column groups they hold (k_coarse_proj<double> spent 37 us
+            // a step at one site a CTA with two warps, most of it on one FP64 pipe of four)
+            int ks = 1;
+            if (std::is_same<T, double>::value && lsw)
+                for (int q : {2, 3, 4, 5, 6, 8, 10, 12, 15, 20})
+                    if (q * rows <= F64_ROW_THREADS) ks = q;
+            const size_t smem = sizeof(ClusterSmem<T>) + (vs ? slice_bytes<T>(ms, rows) : 0) + proj_bytes<T>(k) +
+                                (ks > 1 ? (size_t)ks * rows * sizeof(C2<T>) : 0);
+            if (smem > SMEM_LIMIT) continue;
+            const int thr = (std::is_same<T, double>::value && lsw ? std::max(threads, F64_ROW_THREADS) : threads) + 32 * lsw;
             cudaLaunchConfig_t cfg{};
             cudaLaunchAttribute attr[1];
             attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1466,6 +1666,7 @@ mg_status geometry_uncached(long nsite, int ms, int k, int dev, Geometry& g) {
             g.threads = thr;
             g.vs = vs;
             g.lsw = lsw;
+            g.ks = ks;
             g.smem = smem;
             // FP32 push mode: room for the shared FP16 blocks (used when the handle
             // streams the FP16 operator), if the number of resident clusters holds
@@ -1531,6 +1732,7 @@ mg_status launch_coarse_proj(const CoopArgs<T>& args_in, cudaStream_t s) {
     a.spc = g.spc;
     a.vs = g.vs;
     a.lsw = g.lsw;
+    a.ks = g.ks;
     a.flow = g.lsw;  // push mode
     a.ash = (g.ash && a.Ah) ? 1 : 0;
     cudaLaunchConfig_t cfg{};
