@@ -43,6 +43,13 @@ constexpr int WILSON_COLS = 2000;
 constexpr int WILSON_SHAPES[] = {64, 128, 256, WILSON_TILE + 4, WILSON_TILE + 8, WILSON_COLS + 2, WILSON_COLS + 4};
 constexpr int STENCIL_F32_SHAPES[] = {4, 8, 16, 24, 32};
 constexpr int STENCIL_LR_F32_SHAPES[] = {4, 8, 12, 16};
+// FP64 stencils of fewer sites than this take one CTA a site, its columns split over the
+// warps.  An FP64 instruction of a warp holds its scheduler for 64 cycles, so a site's
+// time is its instructions on the busiest scheduler: a quarter of them when four warps
+// share it.  With a CTA's worth of sites for every SM the eight-site blocks use as many
+// schedulers and need fewer instructions.  Measured: the dense stencil on 20 x 12 sites
+// 24.8 us in eight-site blocks, 7.7 us so; the factored one on 16 x 16 sites 6.5 us.
+constexpr long F64_SPLIT_SITES = 2048;
 
 // ---------------------------------------------------------------- wilson ----
 // y = D x, D^+ x (dagger), or y = b - D x when b != nullptr.  Section 2.

@@ -183,6 +183,59 @@ __global__ void __launch_bounds__(LR_SPB* N) k_stencil_lr(C2<T>* __restrict__ y,
 }
 
 
+// FP64, one CTA of four warps a site (F64_SPLIT_SITES): warp d forms t = R x_nbr of hop
+// direction d + 1 (lane (i, p) three columns of rank i, eight lanes a product), adds
+// Q t to its quarter of the self block's columns, and the four warps' sums are added in
+// order, each real component on its own thread.  Bound by the FP64 pipe and three
+// dependent phases: 6.5 us an apply on 16 x 16 sites.
+__global__ void __launch_bounds__(128) k_stencil_lr_f64_site(double2* __restrict__ y, const double2* __restrict__ x,
+                                                             const double2* __restrict__ F,
+                                                             const double2* __restrict__ b, int Nx, int Nt,
+                                                             int dagger, Gate g) {
+    if (!gate_open(g)) return;
+    __shared__ double2 xs[N], ps[4][N];
+    const int lane = threadIdx.x & 31, d = threadIdx.x >> 5;
+    const long s = blockIdx.x;
+    const int xx = (int)(s % Nx), t = (int)(s / Nx);
+    const long nb = d == 0 ? ((xx + 1 == Nx) ? s - xx : s + 1)
+                    : d == 1 ? ((xx == 0) ? s + Nx - 1 : s - 1)
+                    : d == 2 ? ((t + 1 == Nt) ? (long)xx : s + Nx)
+                             : ((t == 0) ? s + (long)Nx * (Nt - 1) : s - Nx);
+    const double2* Fs = F + s * (long)LR_SITE;
+    const double2* Qd = Fs + N * N + d * LR_BLOCK;
+    const int i = lane >> 3, p = lane & 7;
+    auto flipped = [&](double2 v, int l) { return dagger && l >= N / 2 ? cneg(v) : v; };
+    if (threadIdx.x < N) xs[threadIdx.x] = flipped(x[s * N + threadIdx.x], threadIdx.x);
+    double2 tv = make_double2(0.0, 0.0);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const int l = 3 * p + c;
+        tv = cfma(__ldg(Qd + LR_RANK * N + i * N + l), flipped(x[nb * N + l], l), tv);
+    }
+    // eight lanes a product: half of them keep the real, half the imaginary part
+    double w = ((lane & 4) ? tv.y : tv.x) + __shfl_xor_sync(0xffffffffu, (lane & 4) ? tv.x : tv.y, 4);
+    w += __shfl_xor_sync(0xffffffffu, w, 2);
+    w += __shfl_xor_sync(0xffffffffu, w, 1);
+    __syncthreads();
+    double2 acc = make_double2(0.0, 0.0);
+    const int k = lane < N ? lane : N - 1;
+#pragma unroll
+    for (int c = 0; c < N / 4; ++c) acc = cfma(__ldg(Fs + (d * (N / 4) + c) * N + k), xs[d * (N / 4) + c], acc);
+#pragma unroll
+    for (int q = 0; q < LR_RANK; ++q)
+        acc = cfma(__ldg(Qd + q * N + k),
+                   make_double2(__shfl_sync(0xffffffffu, w, 8 * q), __shfl_sync(0xffffffffu, w, 8 * q + 4)), acc);
+    if (lane < N) ps[d][lane] = acc;
+    __syncthreads();
+    if (threadIdx.x < 2 * N) {
+        const double* q = reinterpret_cast<const double*>(ps) + threadIdx.x;
+        double v = (q[0] + q[2 * N]) + (q[4 * N] + q[6 * N]);
+        if (dagger && (int)threadIdx.x >= N) v = -v;
+        if (b) v = reinterpret_cast<const double*>(b + s * N)[threadIdx.x] - v;
+        reinterpret_cast<double*>(y + s * N)[threadIdx.x] = v;
+    }
+}
+
 // FP32 (bound by HBM): one thread per PAIR of dof rows (12 per site), so every
 // operator load is a 16-byte vector of two rows (Q, the self block) or two
 // columns (R); sites spread evenly over one block per SM and wave, as in the
@@ -299,6 +352,11 @@ void launch_stencil_lr(C2<T>* y, const C2<T>* x, const C2<T>* F, const C2<T>* b,
         const unsigned grid = (unsigned)((nsite + spb - 1) / spb);
         k_stencil_lr_f32<<<grid, spb * LRF_TPS, 0, s>>>(y, x, F, b, Nx, Nt, spb, dagger ? 1 : 0, g);
     } else {
+        if (nsite < F64_SPLIT_SITES) {
+            k_stencil_lr_f64_site<<<(unsigned)nsite, 128, 0, s>>>(y, x, F, b, Nx, Nt, dagger ? 1 : 0, g);
+            count_launch();
+            return;
+        }
         const unsigned grid = (unsigned)((nsite + LR_SPB - 1) / LR_SPB);
         k_stencil_lr<T><<<grid, LR_SPB * N, 0, s>>>(y, x, F, b, Nx, Nt, dagger ? 1 : 0, g);
     }
