@@ -48,6 +48,45 @@ __device__ __forceinline__ C2<T> bblock_sum(C2<T> v, C2<T>* sm) {
     return r;
 }
 
+// Sums over the block of CH complex values a thread holds in acc: value c is returned
+// (valid in threads 2c: real part, 2c + 1: imaginary part, in *out).  A warp's butterfly
+// halves the values it carries at each stage (2 CH - 1 + log2(32 / 2 CH) additions a
+// lane instead of 10 CH), which matters most in FP64, where an addition of a warp holds
+// its scheduler for 64 cycles; the warps' sums are added in warp order.  k_bgram took
+// 66 ms of a 256^2 solve of 64 right-hand sides, 45 ms so (FP64, 131072 entries x 64:
+// 396 us a launch; FP32: 27 us).
+template <typename T, int CH>
+__device__ __forceinline__ T bblock_sums(const C2<T> (&acc)[CH], T (*sm)[2 * CH]) {
+    constexpr int NVAL = 2 * CH;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    T v[NVAL];
+#pragma unroll
+    for (int c = 0; c < CH; ++c) {
+        v[2 * c] = acc[c].x;
+        v[2 * c + 1] = acc[c].y;
+    }
+    int idx = 0;  // the value this lane ends with
+#pragma unroll
+    for (int half = NVAL / 2, o = 16; half > 0; half >>= 1, o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int i = 0; i < half; ++i) {
+            const T send = up ? v[i] : v[i + half];
+            v[i] = (up ? v[i + half] : v[i]) + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+        idx += up ? half : 0;
+    }
+#pragma unroll
+    for (int o = 16 / NVAL; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    __syncthreads();
+    if ((lane & (32 / NVAL - 1)) == 0) sm[warp][idx] = v[0];
+    __syncthreads();
+    T r = 0;
+    if (threadIdx.x < NVAL)
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) r += sm[w][threadIdx.x];
+    return r;
+}
+
 // true in every thread of the last chunk block of right-hand side r
 __device__ __forceinline__ bool blast_chunk(unsigned* ticket) {
     __shared__ bool am_last;
@@ -73,7 +112,24 @@ __device__ __forceinline__ C2<T> bsum_chunks(const C2<T>* part_r, int i) {
 }
 
 constexpr int BT = 256;      // threads of the batched BLAS kernels
-constexpr int BGRAM_CH = 8;  // inner products per pass over the vector
+
+// CH inner products of the vectors V[i0 + c], c < cnt, with w: their chunk partials
+template <typename T, int CH>
+__device__ __forceinline__ void bgram_chunk(const C2<T>* __restrict__ V, long ldv, int i0, int cnt,
+                                            const C2<T>* __restrict__ w, long n, C2<T>* part, T (*sm)[2 * CH]) {
+    const long stride = (long)gridDim.x * BT;
+    C2<T> acc[CH];
+#pragma unroll
+    for (int c = 0; c < CH; ++c) acc[c] = mk<T>(0, 0);
+    for (long e = (long)blockIdx.x * BT + threadIdx.x; e < n; e += stride) {
+        const C2<T> we = w[e];
+#pragma unroll
+        for (int c = 0; c < CH; ++c)
+            if (c < cnt) acc[c] = cfmac(V[(long)(i0 + c) * ldv + e], we, acc[c]);
+    }
+    const T r = bblock_sums<T, CH>(acc, sm);
+    if ((int)threadIdx.x < 2 * cnt) reinterpret_cast<T*>(part + i0)[threadIdx.x] = r;
+}
 
 template <typename T>
 __global__ void __launch_bounds__(BT) k_bgram(double2* __restrict__ out, long os, const C2<T>* __restrict__ V,
@@ -82,31 +138,17 @@ __global__ void __launch_bounds__(BT) k_bgram(double2* __restrict__ out, long os
                                               int max_chunks, unsigned* ticket, Gate g) {
     const int r = blockIdx.y;
     if (!gate_open(g, r)) return;
-    __shared__ C2<T> sm[BT / 32];
+    __shared__ T sm8[BT / 32][16];
+    __shared__ T sm2[BT / 32][4];
     int cnt = nd + (ndd ? ndd[r * nds] : 0);
     if (cnt > RED_MAXD) cnt = RED_MAXD;
     const C2<T>* Vr = V + r * vr;
     const C2<T>* wv = w + r * wr;
     C2<T>* part_r = partial + (size_t)r * max_chunks * RED_MAXD;
-    const long stride = (long)gridDim.x * BT;
-    const long e0 = (long)blockIdx.x * BT + threadIdx.x;
-    for (int i0 = 0; i0 < cnt; i0 += BGRAM_CH) {
-        C2<T> acc[BGRAM_CH];
-#pragma unroll
-        for (int c = 0; c < BGRAM_CH; ++c) acc[c] = mk<T>(0, 0);
-        for (long e = e0; e < n; e += stride) {
-            const C2<T> we = wv[e];
-#pragma unroll
-            for (int c = 0; c < BGRAM_CH; ++c)
-                if (i0 + c < cnt) acc[c] = cfmac(Vr[(long)(i0 + c) * ldv + e], we, acc[c]);
-        }
-#pragma unroll
-        for (int c = 0; c < BGRAM_CH; ++c)
-            if (i0 + c < cnt) {
-                const C2<T> v = bblock_sum<T>(acc[c], sm);
-                if (threadIdx.x == 0) part_r[(size_t)blockIdx.x * RED_MAXD + i0 + c] = v;
-            }
-    }
+    C2<T>* part = part_r + (size_t)blockIdx.x * RED_MAXD;
+    int i0 = 0;
+    for (; cnt - i0 > 2; i0 += 8) bgram_chunk<T, 8>(Vr, ldv, i0, min(8, cnt - i0), wv, n, part, sm8);
+    if (i0 < cnt) bgram_chunk<T, 2>(Vr, ldv, i0, cnt - i0, wv, n, part, sm2);
     if (blast_chunk(ticket + r)) {
         __threadfence();
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
