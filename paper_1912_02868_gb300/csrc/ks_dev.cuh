@@ -92,5 +92,126 @@ __device__ inline void ks_push_dev(KState* ks, int jh) {
     ks->scale = (hn > 0.0) ? 1.0 / hn : 0.0;
 }
 
+
+// Start of a cycle from a vector of squared norm nrm2v, by one warp
+__device__ inline void ks_start_dev(KState* ks, double nrm2v, double tol_rel, double nb2v) {
+    const double beta = sqrt(fmax(nrm2v, 0.0));
+    const double tol_abs = tol_rel * sqrt(fmax(nb2v, 0.0));
+    const int lane = threadIdx.x & 31;  // one warp: lane 0 writes the scalars
+    for (int i = lane; i < KLD; i += 32) ks->c[i] = ks->g[i] = make_double2(i == 0 ? beta : 0.0, 0.0);
+    if (lane != 0) return;
+    ks->beta = beta;
+    ks->tol_abs = tol_abs;
+    ks->res = beta;
+    ks->nrot = 0;
+    ks->j = 0;
+    ks->j0 = 0;
+    ks->conv = (beta <= tol_abs) ? 1 : 0;
+    ks->breakdown = 0;
+    ks->err = 0;
+    ks->step_gate = (!ks->conv && beta > 0.0) ? 0 : -1;
+    ks->scale = beta > 0.0 ? 1.0 / beta : 0.0;
+    ks->scale_gate = 0;
+}
+// ks_push_dev by one warp: the column and the earlier rotations are read
+// into shared memory at once, so that the serial chain of rotations (lane 0) waits for
+// no dependent global load, and the column's zeros are written by all lanes.
+struct PushScratch {
+    double2 col[KLD];
+    double2 rs[NROT];
+    double rc[NROT];
+    short ra[NROT], rb[NROT];
+};
+__device__ inline void ks_push_warp(KState* ks, int jh, PushScratch& S) {
+    double2 *col = S.col, *rs = S.rs;
+    double* rc = S.rc;
+    short *ra = S.ra, *rb = S.rb;
+    const int lane = threadIdx.x & 31, j = jh;
+    if (ks->step_gate != jh) return;
+    const int nr = ks->nrot;
+    for (int t = lane; t < nr; t += 32) {
+        rc[t] = ks->rc[t];
+        rs[t] = ks->rs[t];
+        ra[t] = ks->ra[t];
+        rb[t] = ks->rb[t];
+    }
+    for (int i = lane; i <= j; i += 32) col[i] = cadd(ks->hA[i], ks->hB[i]);
+    for (int i = j + 2 + lane; i < KLD; i += 32) col[i] = z0();
+    const double hn2 = fmax(ks->hn2, 0.0), hn = sqrt(hn2), inv = hn > 0.0 ? 1.0 / hn : 0.0;
+    if (lane == 0) col[j + 1] = make_double2(hn, 0.0);
+    const double2 gj = ks->g[j];
+    const double tol_abs = ks->tol_abs;
+    __syncwarp();
+    for (int i = lane; i < KLD; i += 32) ks->H[i + KLD * j] = col[i];
+    __syncwarp();
+    if (lane == 0) {
+        for (int t = 0; t < nr; ++t) rot_apply(rc[t], rs[t], col[ra[t]], col[rb[t]]);
+        double c;
+        double2 sn, r;
+        givens(col[j], col[j + 1], c, sn, r);
+        col[j] = r;
+        col[j + 1] = z0();
+        ks->rc[nr] = c;
+        ks->rs[nr] = sn;
+        ks->ra[nr] = (short)j;
+        ks->rb[nr] = (short)(j + 1);
+        ks->nrot = nr + 1;
+        double2 g0 = gj, g1 = ks->g[j + 1];
+        rot_apply(c, sn, g0, g1);
+        ks->g[j] = g0;
+        ks->g[j + 1] = g1;
+        const double res = cabsd(g1);
+        const int conv = res <= tol_abs ? 1 : 0, brk = hn == 0.0 ? 1 : 0;
+        ks->res = res;
+        ks->j = j + 1;
+        ks->breakdown = brk;
+        ks->conv = conv;
+        ks->step_gate = (conv || brk || j + 1 >= KMAX) ? -1 : j + 1;
+        ks->scale_gate = (hn > 0.0) ? j + 1 : -1;
+        ks->scale = inv;
+    }
+    __syncwarp();
+    for (int i = lane; i < KLD; i += 32) ks->R[i + KLD * j] = col[i];
+}
+// Back substitution R d = g over the first jj <= MAXJ columns, by one warp: R is read
+// into shared memory at once, the lanes form the reciprocals of their pivots together
+// (a zero pivot gives d_i = 0 and *err = 2), and each column then costs a product, a
+// broadcast and a subtraction on the serial chain.  k_bks_finish for 64 right-hand
+// sides: 39 us with R and the divides on one thread, 24 us so.
+template <int MAXJ>
+__device__ inline void solve_upper(const double2* R, const double2* g, double2* d, int jj, int* err) {
+    __shared__ double2 Rs[MAXJ * (MAXJ + 1) / 2];  // column i: rows 0..i at i (i + 1) / 2
+    const int lane = threadIdx.x & 31;
+    for (int i = 0; i < jj; ++i)
+        for (int r = lane; r <= i; r += 32) Rs[i * (i + 1) / 2 + r] = R[r + KLD * i];
+    __syncwarp();
+    double2 acc[2], inv[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int r = lane + 32 * h;
+        acc[h] = inv[h] = z0();
+        if (r < jj) {
+            acc[h] = g[r];
+            const double2 piv = Rs[r * (r + 1) / 2 + r];
+            if (piv.x == 0.0 && piv.y == 0.0) {
+                if (err) *err = 2;
+            } else {
+                inv[h] = cdiv(make_double2(1.0, 0.0), piv);
+            }
+        }
+    }
+    for (int i = jj - 1; i >= 0; --i) {
+        const double2* Ri = Rs + i * (i + 1) / 2;
+        double2 di = i >= 32 ? cmul(acc[1], inv[1]) : cmul(acc[0], inv[0]);
+        di.x = __shfl_sync(0xffffffffu, di.x, i & 31);
+        di.y = __shfl_sync(0xffffffffu, di.y, i & 31);
+        if (lane == (i & 31)) d[i] = di;
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            if (lane + 32 * h < i) acc[h] = csub(acc[h], cmul(Ri[lane + 32 * h], di));
+    }
+    __syncwarp();
+}
+
 }  // namespace ksd
 }  // namespace mg

@@ -84,6 +84,20 @@ constexpr long KS_INTS = (long)(sizeof(KState) / sizeof(int));
 constexpr long KS_DBLS = (long)(sizeof(KState) / sizeof(double));
 constexpr long KS_CPLX = (long)(sizeof(KState) / sizeof(double2));
 
+// Arnoldi vector work as cluster kernels (arnoldi.cu), for vectors within their sizes;
+// false, with nothing enqueued, for others.
+// CGS2 of V[j + 1] against V[0..j] (rows of n), its norm, the push of column j into
+// ks and the normalisation; gated
+template <typename T>
+bool launch_arnoldi(C2<T>* V, long n, int j, KState* ks, Gate g, cudaStream_t s);
+// ks started from ||f|| with tolerance 0, v0 = f / ||f||
+template <typename T>
+bool launch_krylov_start(C2<T>* v0, const C2<T>* f, long n, KState* ks, cudaStream_t s);
+// ks finished (at most `steps` columns), x = V d (or x += V d), r = V rho unless null
+template <typename T>
+bool launch_finish_update(C2<T>* x, C2<T>* r, const C2<T>* V, long n, int steps, KState* ks, bool accumulate,
+                          cudaStream_t s);
+
 // GMRES-DR restart from the finished cycle in ks (harmonic Ritz vectors).
 mg_status dr_restart(const KState* ks, DRState* dr, int k, cudaStream_t s);
 // *out = 1 / sqrt(*in)

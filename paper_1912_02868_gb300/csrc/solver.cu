@@ -62,6 +62,7 @@ void arnoldi_step(Handle& H, OpFn&& op, C2<T>* V, long n, KState* ks, int jh, cu
     const Gate g{MG_DEVF(ks, int, step_gate), jh};
     C2<T>* w = V + (long)(jh + 1) * n;
     op(w, g);
+    if (launch_arnoldi<T>(V, n, jh, ks, g, s)) return;
     double2* hA = MG_DEVF(ks, double2, hA);
     double2* hB = MG_DEVF(ks, double2, hB);
     launch_gram<T>(hA, V, n, jh + 1, w, n, H.red, g, s);
@@ -79,19 +80,23 @@ void smoother(Handle& H, int l, Level<T>& L, const C2<T>* f, C2<T>* x, bool accu
     const long n = L.n;
     double* t = MG_DEVF(H.sc, double, tmp);
     KState* ks = L.ks;
-    launch_norm2<T>(t, f, n, H.red, Gate{}, s);
-    ks_start(ks, t, 0.0, t, s);
-    launch_scale<T>(L.sV, f, MG_DEVF(ks, double, scale), n, Gate{MG_DEVF(ks, int, scale_gate), 0}, s);
+    if (!launch_krylov_start<T>(L.sV, f, n, ks, s)) {
+        launch_norm2<T>(t, f, n, H.red, Gate{}, s);
+        ks_start(ks, t, 0.0, t, s);
+        launch_scale<T>(L.sV, f, MG_DEVF(ks, double, scale), n, Gate{MG_DEVF(ks, int, scale_gate), 0}, s);
+    }
     for (int jh = 0; jh < H.p.smooth_steps; ++jh) {
         const C2<T>* in = L.sV + (long)jh * n;
         arnoldi_step<T>(H, [&](C2<T>* w, Gate g) { L.apply(w, in, nullptr, false, g, s); }, L.sV, n, ks, jh, s);
     }
-    ks_finish(ks, s);
-    launch_axpy_multi<T>(x, L.sV, n, 0, MG_DEVF(ks, int, j), MG_DEVF(ks, double2, d), 1.0, !accumulate, n, nullptr,
-                         H.red, Gate{}, s);
-    if (r_out)
-        launch_axpy_multi<T>(r_out, L.sV, n, 1, MG_DEVF(ks, int, j), MG_DEVF(ks, double2, rho), 1.0, true, n,
-                             nullptr, H.red, Gate{}, s);
+    if (!launch_finish_update<T>(x, r_out, L.sV, n, H.p.smooth_steps, ks, accumulate, s)) {
+        ks_finish(ks, s);
+        launch_axpy_multi<T>(x, L.sV, n, 0, MG_DEVF(ks, int, j), MG_DEVF(ks, double2, d), 1.0, !accumulate, n, nullptr,
+                             H.red, Gate{}, s);
+        if (r_out)
+            launch_axpy_multi<T>(r_out, L.sV, n, 1, MG_DEVF(ks, int, j), MG_DEVF(ks, double2, rho), 1.0, true, n,
+                                 nullptr, H.red, Gate{}, s);
+    }
     H.st.mvps[l] += H.p.smooth_steps;
 }
 
