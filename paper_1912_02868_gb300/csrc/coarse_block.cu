@@ -10,7 +10,8 @@
 //       single-right-hand-side cluster kernel) and pushes column j into the FP64
 //       least squares of each right-hand side;
 //   S3  v_{j+1} = (w - V h2) / h_{j+1,j}.
-// Two forms run them.  The cycle kernel (k_cb_cycle) keeps every CTA of the
+// Three forms run them.  Chunks of at most 16 sites (up to 2432 sites x tiles on 152
+// SMs) take the kernel of coarse_cycle.cu.  The cycle kernel here (k_cb_cycle) keeps every CTA of the
 // block resident (cooperative launch) and runs all steps of a GMRES cycle: the
 // CTAs of a tile meet at a bounded tile barrier after each phase, and each CTA
 // adds the chunk partials of its right-hand sides itself.  The step kernels
@@ -19,77 +20,24 @@
 // The step gate of a right-hand side is double-buffered by step parity: the
 // push of step j writes the gate that step j + 1 reads, while every CTA of step
 // j reads the buffer of step j.  The basis rows are V[i][r][n] (FP32).
-#include <cuda_bf16.h>
-#include <cuda_fp16.h>
-
 #include <algorithm>
 #include <mutex>
 #include <vector>
 
-#include "batch.cuh"
-#include "coarse_block.cuh"
-#include "ks_dev.cuh"
+#include "coarse_block_dev.cuh"
 
 namespace mg {
 
+using namespace cbdev;
+
 namespace {
 
-constexpr int NDOF = 24;
-constexpr int TILE_WORDS = 64;
-constexpr int SITE_WORDS = 5 * 9 * TILE_WORDS;
-constexpr int MAXI = MSMAX + 1;  // basis vectors of a cycle
 #ifndef CB_APPLY_MT
 #define CB_APPLY_MT 3  // output tiles per apply task of the cycle kernel (1 or 3)
 #endif
 #ifndef CB_COOP_MINB
 #define CB_COOP_MINB 1  // resident cycle-kernel CTAs per SM the register budget is sized for
 #endif
-
-template <bool F16>
-__device__ __forceinline__ unsigned pk(float re, float im) {
-    if constexpr (F16) {
-        const __half2 h = __floats2half2_rn(re, im);
-        return *reinterpret_cast<const unsigned*>(&h);
-    } else {
-        const __nv_bfloat162 h = __floats2bfloat162_rn(re, im);
-        return *reinterpret_cast<const unsigned*>(&h);
-    }
-}
-template <bool F16>
-__device__ __forceinline__ float2 upk(unsigned u) {
-    if constexpr (F16) return __half22float2(*reinterpret_cast<const __half2*>(&u));
-    else return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u));
-}
-template <bool F16>
-__device__ __forceinline__ void mma(float (&c)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
-    if constexpr (F16)
-        asm volatile(
-            "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-            "{%0,%1,%2,%3};\n"
-            : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-            : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-    else
-        asm volatile(
-            "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-            "{%0,%1,%2,%3};\n"
-            : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-            : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-__device__ __forceinline__ unsigned embed(unsigned w, int p) {
-    return p ? __byte_perm(w, 0u, 0x1032) : (w ^ 0x80000000u);
-}
-// neighbour site in direction d (self, +x, -x, +t, -t), periodic; 32-bit index
-// arithmetic (a coarse grid has far fewer than 2^31 sites)
-__device__ __forceinline__ int nbr_of(int s, int d, int Nx, int Nt) {
-    const int t = s / Nx, xx = s - t * Nx;
-    switch (d) {
-        case 0: return s;
-        case 1: return (xx + 1 == Nx) ? s - xx : s + 1;
-        case 2: return (xx == 0) ? s + Nx - 1 : s - 1;
-        case 3: return (t + 1 == Nt) ? xx : s + Nx;
-        default: return (t == 0) ? s + Nx * (Nt - 1) : s - Nx;
-    }
-}
 
 __device__ __forceinline__ float2 warp_sum2(float2 v) {
 #pragma unroll
@@ -161,73 +109,10 @@ struct CBSmem {
 // (sized at launch, so larger coarse grids can take larger chunks)
 struct CBCycleSmem {
     float2 hs[NB_TILE * CB_WPR][MAXI];
-    float2 h1[NB_TILE][MAXI];      // chunk 0: first-pass products kept for the push
-    float hn[NB_TILE];
-    // chunk 0: the least squares of each right-hand side during the cycle (FP64):
-    // rotations, the rotated right-hand side, the tolerance, and a column
-    double rc[NB_TILE][MSMAX];
-    double2 rs[NB_TILE][MSMAX];
-    double2 g[NB_TILE][MSMAX + 1];
-    double2 col[NB_TILE][MAXI + 1];
-    double tol[NB_TILE];
+    CBPush p;
     WarpRed red[NB_TILE * CB_WPR];
     uint4 abuf[NB_TILE * CB_WPR][SITE_WORDS / 4];  // each warp's staged operator tiles of one site
 };
-
-// Column jh of right-hand side r's least squares (the cycle kernel's push): the
-// column h1 + h2 with subdiagonal hn, rotated by the cycle's earlier rotations
-// (kept in shared memory, so no step waits on a dependent global load), a new
-// rotation, the rotated right-hand side, the residual estimate and the gates.
-// The state in global memory receives what the cycle's finish reads (H, R, g,
-// rotations, j, res, conv) without being read back.
-__device__ __forceinline__ void push_cycle(const CBArgs& a, CBCycleSmem& S, int l, int r, int jh, const float2* h2) {
-    KState* ks = a.ks + r;
-    double2* col = S.col[l];
-    for (int i = 0; i <= jh; ++i) col[i] = make_double2((double)S.h1[l][i].x + (double)h2[i].x,
-                                                        (double)S.h1[l][i].y + (double)h2[i].y);
-    const double hn = (double)S.hn[l];
-    col[jh + 1] = make_double2(hn, 0.0);
-    double2* Hc = ks->H + KLD * jh;
-    double2* Rc = ks->R + KLD * jh;
-    for (int i = 0; i <= jh + 1; ++i) Hc[i] = col[i];
-    for (int i = jh + 2; i < KLD; ++i) {
-        Hc[i] = make_double2(0.0, 0.0);
-        Rc[i] = make_double2(0.0, 0.0);
-    }
-    double2 p = col[0];
-    for (int t = 0; t < jh; ++t) {
-        double2 q = col[t + 1];
-        ksd::rot_apply(S.rc[l][t], S.rs[l][t], p, q);
-        Rc[t] = p;
-        p = q;
-    }
-    double cc;
-    double2 ss, rr;
-    ksd::givens(p, col[jh + 1], cc, ss, rr);
-    Rc[jh] = rr;
-    Rc[jh + 1] = make_double2(0.0, 0.0);
-    S.rc[l][jh] = cc;
-    S.rs[l][jh] = ss;
-    ks->rc[jh] = cc;
-    ks->rs[jh] = ss;
-    ks->ra[jh] = (short)jh;
-    ks->rb[jh] = (short)(jh + 1);
-    ksd::rot_apply(cc, ss, S.g[l][jh], S.g[l][jh + 1]);
-    ks->g[jh] = S.g[l][jh];
-    ks->g[jh + 1] = S.g[l][jh + 1];
-    const double res = ksd::cabsd(S.g[l][jh + 1]);
-    const int conv = res <= S.tol[l] ? 1 : 0, brk = hn == 0.0 ? 1 : 0;
-    const int next = (conv || brk || jh + 1 >= KMAX) ? -1 : jh + 1;
-    ks->nrot = jh + 1;
-    ks->res = res;
-    ks->j = jh + 1;
-    ks->conv = conv;
-    ks->breakdown = brk;
-    ks->step_gate = next;
-    ks->scale_gate = hn > 0.0 ? jh + 1 : -1;
-    ks->scale = hn > 0.0 ? 1.0 / hn : 0.0;
-    a.gbuf[((jh + 1) & 1) * a.nbp + r] = next;
-}
 
 // slots 0..jh (and, with norm, slot CB_PB - 1) of right-hand side r summed over
 // the chunks: lanes over the chunks in a fixed order, then lane_sums.  Lane i
@@ -274,7 +159,7 @@ __device__ __forceinline__ void phase_apply(const CBArgs& a, int jh, int r0, int
                                             float2 (*ws)[CB_MAXSPC * NDOF], int nwarps) {
     constexpr int NT = 3 / MT;  // tasks per site
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int gq = lane >> 2, t = lane & 3, p = gq & 1;
+    const int gq = lane >> 2, t = lane & 3;
     const float2* X = a.V + (long)jh * a.row;
     float2* Wt = a.V + (long)(jh + 1) * a.row;
     for (int task = warp; task < ns * NT; task += nwarps) {
@@ -285,11 +170,11 @@ __device__ __forceinline__ void phase_apply(const CBArgs& a, int jh, int r0, int
         for (int m = 0; m < MT; ++m)
 #pragma unroll
             for (int i = 0; i < 4; ++i) acc[m][i] = 0.f;
-        const uint4* A4 = reinterpret_cast<const uint4*>(a.Af) + (long)s * (SITE_WORDS / 4) + (gq >> 1) * 4 + t +
-                          mt0 * 3 * (TILE_WORDS / 4);
+        const uint2* A2 = reinterpret_cast<const uint2*>(a.Af) + (long)s * (SITE_WORDS / 2) + lane +
+                          mt0 * 3 * (TILE_WORDS / 2);
         const float2* Xr = X + (long)(r0 + gq) * a.n;
         float2 xv[3][2];
-        uint4 aw[MT][3];
+        uint2 aw[MT][3];
         auto load = [&](int d) {
             const float2* xn = Xr + (long)nbr_of(s, d, a.Nx, a.Nt) * NDOF;
 #pragma unroll
@@ -297,14 +182,14 @@ __device__ __forceinline__ void phase_apply(const CBArgs& a, int jh, int r0, int
                 xv[kt][0] = __ldcg(xn + 8 * kt + t);
                 xv[kt][1] = __ldcg(xn + 8 * kt + t + 4);
 #pragma unroll
-                for (int m = 0; m < MT; ++m) aw[m][kt] = __ldg(A4 + (d * 9 + m * 3 + kt) * (TILE_WORDS / 4));
+                for (int m = 0; m < MT; ++m) aw[m][kt] = __ldg(A2 + (d * 9 + m * 3 + kt) * (TILE_WORDS / 2));
             }
         };
         load(0);
 #pragma unroll 1
         for (int d = 0; d < 5; ++d) {
             float2 xc[3][2];
-            uint4 ac[MT][3];
+            uint2 ac[MT][3];
 #pragma unroll
             for (int kt = 0; kt < 3; ++kt) {
                 xc[kt][0] = xv[kt][0];
@@ -321,22 +206,18 @@ __device__ __forceinline__ void phase_apply(const CBArgs& a, int jh, int r0, int
                 const unsigned l0 = pk<F16>(x0.x - f0.x, x0.y - f0.y), l1 = pk<F16>(x1.x - f1.x, x1.y - f1.y);
 #pragma unroll
                 for (int m = 0; m < MT; ++m) {
-                    const uint4 w = ac[m][kt];
-                    const unsigned av[4] = {embed(w.x, p), embed(w.y, p), embed(w.z, p), embed(w.w, p)};
+                    const uint2 w = ac[m][kt];
+                    const unsigned av[4] = {embed(w.x, 0), embed(w.x, 1), embed(w.y, 0), embed(w.y, 1)};
                     mma<F16>(acc[m], av, h0, h1);
                     mma<F16>(acc[m], av, l0, l1);
                 }
             }
         }
-        // lane (gq, t) holds component p of outputs gq / 2 and gq / 2 + 4 of
-        // right-hand sides 2t, 2t + 1; lane ^ 4 holds the other component
+        // lane (gq, t) holds output row gq of right-hand sides 2t, 2t + 1
 #pragma unroll
         for (int m = 0; m < MT; ++m) {
-            const float s0v = p ? acc[m][0] : acc[m][2], s1v = p ? acc[m][1] : acc[m][3];
-            const float o0 = __shfl_xor_sync(0xffffffffu, s0v, 4), o1 = __shfl_xor_sync(0xffffffffu, s1v, 4);
-            const int row = 8 * (mt0 + m) + (gq >> 1) + (p ? 4 : 0);
-            const float2 v0 = p ? make_float2(o0, acc[m][2]) : make_float2(acc[m][0], o0);
-            const float2 v1 = p ? make_float2(o1, acc[m][3]) : make_float2(acc[m][1], o1);
+            const int row = 8 * (mt0 + m) + gq;
+            const float2 v0 = make_float2(acc[m][0], acc[m][2]), v1 = make_float2(acc[m][1], acc[m][3]);
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
                 const int rl = 2 * t + q;
@@ -356,7 +237,7 @@ template <bool F16>
 __device__ __forceinline__ void phase_apply_staged(const CBArgs& a, int jh, int r0, int s0, int ns, unsigned wmask,
                                                    float2* ws, int wst, uint4* abuf, int nwarps) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int gq = lane >> 2, t = lane & 3, p = gq & 1;
+    const int gq = lane >> 2, t = lane & 3;
     const float2* X = a.V + (long)jh * a.row;
     float2* Wt = a.V + (long)(jh + 1) * a.row;
     constexpr int SITE_U4 = SITE_WORDS / 4;  // 720 sixteen-byte pieces
@@ -386,7 +267,7 @@ __device__ __forceinline__ void phase_apply_staged(const CBArgs& a, int jh, int 
         for (int m = 0; m < 3; ++m)
 #pragma unroll
             for (int i = 0; i < 4; ++i) acc[m][i] = 0.f;
-        const uint4* A4 = abuf + (gq >> 1) * 4 + t;
+        const uint2* A2 = reinterpret_cast<const uint2*>(abuf) + lane;
 #pragma unroll
         for (int d = 0; d < 5; ++d) {
 #pragma unroll
@@ -397,8 +278,8 @@ __device__ __forceinline__ void phase_apply_staged(const CBArgs& a, int jh, int 
                 const unsigned l0 = pk<F16>(x0.x - f0.x, x0.y - f0.y), l1 = pk<F16>(x1.x - f1.x, x1.y - f1.y);
 #pragma unroll
                 for (int m = 0; m < 3; ++m) {
-                    const uint4 w = A4[(d * 9 + m * 3 + kt) * (TILE_WORDS / 4)];
-                    const unsigned av[4] = {embed(w.x, p), embed(w.y, p), embed(w.z, p), embed(w.w, p)};
+                    const uint2 w = A2[(d * 9 + m * 3 + kt) * (TILE_WORDS / 2)];
+                    const unsigned av[4] = {embed(w.x, 0), embed(w.x, 1), embed(w.y, 0), embed(w.y, 1)};
                     mma<F16>(acc[m], av, h0, h1);
                     mma<F16>(acc[m], av, l0, l1);
                 }
@@ -406,11 +287,8 @@ __device__ __forceinline__ void phase_apply_staged(const CBArgs& a, int jh, int 
         }
 #pragma unroll
         for (int m = 0; m < 3; ++m) {
-            const float s0v = p ? acc[m][0] : acc[m][2], s1v = p ? acc[m][1] : acc[m][3];
-            const float o0 = __shfl_xor_sync(0xffffffffu, s0v, 4), o1 = __shfl_xor_sync(0xffffffffu, s1v, 4);
-            const int row = 8 * m + (gq >> 1) + (p ? 4 : 0);
-            const float2 v0 = p ? make_float2(o0, acc[m][2]) : make_float2(acc[m][0], o0);
-            const float2 v1 = p ? make_float2(o1, acc[m][3]) : make_float2(acc[m][1], o1);
+            const int row = 8 * m + gq;
+            const float2 v0 = make_float2(acc[m][0], acc[m][2]), v1 = make_float2(acc[m][1], acc[m][3]);
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
                 const int rl = 2 * t + q;
@@ -420,14 +298,6 @@ __device__ __forceinline__ void phase_apply_staged(const CBArgs& a, int jh, int 
             }
         }
     }
-}
-
-// the bits of the tile's right-hand sides whose gate opens step jh
-__device__ __forceinline__ unsigned gate_mask(const int* gate, int r0, int jh) {
-    unsigned m = 0u;
-#pragma unroll
-    for (int q = 0; q < NB_TILE; ++q) m |= (__ldcg(gate + r0 + q) == jh ? 1u : 0u) << q;
-    return m;
 }
 
 // partial sums over the chunk of V^+ w (w in ws) for right-hand side r, one
@@ -748,8 +618,8 @@ __global__ void __launch_bounds__(CB_COOP_THREADS, CB_COOP_MINB) k_cb_cycle(CBAr
     }
     if (c == 0 && warp == NRW && lane < NB_TILE) {  // the least squares as the cycle's start left it
         const KState* ks = a.ks + r0 + lane;
-        for (int i = 0; i <= MSMAX; ++i) S.g[lane][i] = ks->g[i];
-        S.tol[lane] = ks->tol_abs;
+        for (int i = 0; i <= MSMAX; ++i) S.p.g[lane][i] = ks->g[i];
+        S.p.tol[lane] = ks->tol_abs;
     }
     __syncthreads();
     // The push of step jh - 1 (warp NRW of chunk 0) runs while the other warps
@@ -765,8 +635,10 @@ __global__ void __launch_bounds__(CB_COOP_THREADS, CB_COOP_MINB) k_cb_cycle(CBAr
         // phase 1: w = A v_jh, partial sums of V^+ w (speculative for step jh > 0)
         if (rw) phase_apply_staged<F16>(a, jh, r0, s0, ns, spec, wsb, wst, S.abuf[warp], NRW);
         else if (jh > 0 && warp == NRW && c == 0 && lane < NB_TILE &&
-                 __ldcg(a.gbuf + ((jh - 1) & 1) * a.nbp + r0 + lane) == jh - 1)
-            push_cycle(a, S, lane, r0 + lane, jh - 1, S.hs[lane]);  // warp `lane` (part 0) holds h2
+                 __ldcg(a.gbuf + ((jh - 1) & 1) * a.nbp + r0 + lane) == jh - 1) {
+            push_column_entries(S.p, lane, jh - 1, S.hs[lane], 0, 1);  // warp `lane` (part 0) holds h2
+            push_cycle(a, S.p, lane, r0 + lane, jh - 1, -1);
+        }
         __syncthreads();
         CB_STAMP(6);
         if (spec_on) CB_DISPATCH(jh, (phase_gram1<JB>(a, jh, r, slot, s0, ne, e0, es, wsb + rl * wst, S.red[warp])));
@@ -785,7 +657,7 @@ __global__ void __launch_bounds__(CB_COOP_THREADS, CB_COOP_MINB) k_cb_cycle(CBAr
             CB_DISPATCH(jh, (t = chunk_totals<JB>(a.p1, nslot, r, jh, false, nullptr, S.red[warp])));
             if (lane <= jh) {
                 S.hs[warp][lane] = t;
-                if (c == 0 && part == 0) S.h1[rl][lane] = t;
+                if (c == 0 && part == 0) S.p.h1[rl][lane] = t;
             }
             __syncwarp();
             CB_DISPATCH(jh, (phase_update_gram<false, JB>(a, jh, r, slot, s0, ne, e0, es, S.hs[warp], S.red[warp])));
@@ -800,7 +672,7 @@ __global__ void __launch_bounds__(CB_COOP_THREADS, CB_COOP_MINB) k_cb_cycle(CBAr
             CB_DISPATCH(jh, (t = chunk_totals<JB>(a.p2, nslot, r, jh, true, &nrm, S.red[warp])));
             const float hn = subdiag(t, jh, nrm);
             if (lane <= jh) S.hs[warp][lane] = t;
-            if (lane == 0 && part == 0) S.hn[rl] = hn;
+            if (lane == 0 && part == 0) S.p.hn[rl] = hn;
             __syncwarp();
             CB_DISPATCH(jh, (phase_update<JB>(a, jh, r, s0, ne, e0, es, S.hs[warp], hn > 0.f ? 1.f / hn : 0.f)));
         }
@@ -815,8 +687,10 @@ __global__ void __launch_bounds__(CB_COOP_THREADS, CB_COOP_MINB) k_cb_cycle(CBAr
     // the last step's push, when the loop ran to the cycle length (after an early
     // exit every push has run: the exit follows the phase that pushed)
     if (jh == ms && warp == NRW && c == 0 && lane < NB_TILE &&
-        __ldcg(a.gbuf + ((ms - 1) & 1) * a.nbp + r0 + lane) == ms - 1)
-        push_cycle(a, S, lane, r0 + lane, ms - 1, S.hs[lane]);
+        __ldcg(a.gbuf + ((ms - 1) & 1) * a.nbp + r0 + lane) == ms - 1) {
+        push_column_entries(S.p, lane, ms - 1, S.hs[lane], 0, 1);
+        push_cycle(a, S.p, lane, r0 + lane, ms - 1, -1);
+    }
 #ifdef CB_PHASE_CLOCKS
     if (clk && threadIdx.x == 0 && steps > 0)
         printf("cb_cycle phases (ns/step over %d steps, %d chunks): apply %llu, gram1 %llu, bar1 %llu, "
@@ -832,6 +706,7 @@ __global__ void k_cb_gate_init(CBArgs a) {
         a.gbuf[r] = a.ks[r].step_gate;
         a.gbuf[a.nbp + r] = -1;  // no stale index of an earlier cycle can match a step
     }
+    if (r == 0) *a.epoch += CB_TAGS;  // the launch's tags
 }
 
 }  // namespace
@@ -894,7 +769,7 @@ bool cb_geometry_cycle(CBArgs& a, long nsite, int nbp, bool fp16) {
         long nsite;
         int nbp;
         bool fp16, ok;
-        int spc, nchunks;
+        int spc, nchunks, coop, srows;
     };
     static std::mutex mu;
     static std::vector<Entry> cache;
@@ -911,13 +786,14 @@ bool cb_geometry_cycle(CBArgs& a, long nsite, int nbp, bool fp16) {
                 a.spc = e.spc;
                 a.nchunks = e.nchunks;
                 a.nbp = nbp;
-                a.coop = 1;
+                a.coop = e.coop;
+                a.srows = e.srows;
                 return true;
             }
     }
-    const bool ok = cb_geometry_cycle_uncached(a, nsite, nbp, fp16);
+    const bool ok = cb_geometry_chunk(a, nsite, nbp, fp16) || cb_geometry_cycle_uncached(a, nsite, nbp, fp16);
     std::lock_guard<std::mutex> lock(mu);
-    cache.push_back(Entry{dev, nsite, nbp, fp16, ok, ok ? a.spc : 0, ok ? a.nchunks : 0});
+    cache.push_back(Entry{dev, nsite, nbp, fp16, ok, a.spc, a.nchunks, a.coop, a.srows});
     return ok;
 }
 
@@ -969,6 +845,7 @@ void launch_cb_step(const CBArgs& a, int jh, bool fp16, cudaStream_t s) {
 }
 
 mg_status launch_cb_cycle(const CBArgs& a, int ms, bool fp16, long spin, int* err, cudaStream_t s) {
+    if (a.coop == 2) return launch_cb_chunk(a, ms, fp16, spin, err, s);
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;

@@ -31,7 +31,15 @@ struct CBArgs {
     unsigned* bar;       // [nbp / 8][2] tile barrier (count, generation) of the cycle kernel, then
                          // one word that nothing writes (the probe's)
     int spc, nchunks, nbp;
-    int coop;            // 1: geometry of the cycle kernel
+    int coop;            // 1: geometry of the cycle kernel, 2: of the chunk kernel (coarse_cycle.cu)
+    // chunk kernel: tagged partial sums of the two passes [nbp][CB_PB][nchunks], the row
+    // flags of the chunks and the gate word of each tile, the tag base, and the basis rows
+    // a CTA keeps in shared memory
+    ulonglong2 *t1, *t2;
+    unsigned* flags;
+    unsigned long long* gword;
+    unsigned* epoch;
+    int srows;
     int probe;           // test probe: every CTA first waits (bounded) on the word nothing writes
 };
 
@@ -49,5 +57,14 @@ void launch_cb_step(const CBArgs& a, int jh, bool fp16, cudaStream_t s);
 // all ms steps of a cycle in one cooperative launch (cb_geometry_cycle); a tile
 // barrier that waits longer than `spin` polls sets *err
 mg_status launch_cb_cycle(const CBArgs& a, int ms, bool fp16, long spin, int* err, cudaStream_t s);
+
+
+// The chunk kernel (coarse_cycle.cu): geometry (false where it does not fit), the words of
+// t1 or t2 for nbp right-hand sides, the flags of all tiles, and a whole cycle
+bool cb_geometry_chunk(CBArgs& a, long nsite, int nbp, bool fp16);
+size_t cb_chunk_words(int nbp);
+int cb_chunk_flags();
+constexpr unsigned CB_TAGS = 64;  // tags of one launch, at least its steps + 1
+mg_status launch_cb_chunk(const CBArgs& a, int ms, bool fp16, long spin, int* err, cudaStream_t s);
 
 }  // namespace mg

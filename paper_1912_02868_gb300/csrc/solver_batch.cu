@@ -88,6 +88,9 @@ struct BatchWS {
     float2 *ch1 = nullptr, *ch2 = nullptr;  // fused-step reduced products
     unsigned* ctk = nullptr;                // fused-step tickets
     unsigned* cbar = nullptr;               // tile barriers of the cycle kernel
+    ulonglong2* ctw = nullptr;              // chunk kernel: tagged sums of both passes,
+    unsigned* cfl = nullptr;                // row flags, the tag base behind them,
+    unsigned long long* cgw = nullptr;      // and gate words
     bool no_coop = false;                   // the cycle kernel could not be captured: use the step kernels
     int probe = 0;                          // coarse test probe (mg_coarse_solve): a wait that gives up
     long spin = 0;                          // polls of a tile barrier before it gives up (0: default)
@@ -182,6 +185,14 @@ mg_status batch_alloc(Handle& H, int nbp, bool fp16, cudaStream_t s) {
         MG_CUDA_TRY(cudaMemsetAsync(B.ctk, 0, 2 * NB_MAX / NB_TILE * sizeof(unsigned), s));
         MG_TRY(halloc_t(H, &B.cbar, (size_t)2 * NB_MAX / NB_TILE + 1));
         MG_CUDA_TRY(cudaMemsetAsync(B.cbar, 0, (2 * NB_MAX / NB_TILE + 1) * sizeof(unsigned), s));
+        // no word may hold a tag before it is written: all start at zero, the tags above it
+        const size_t words = 2 * cb_chunk_words(nbp), flags = (size_t)cb_chunk_flags() + 1;
+        MG_TRY(halloc_t(H, &B.ctw, words));
+        MG_CUDA_TRY(cudaMemsetAsync(B.ctw, 0, words * sizeof(ulonglong2), s));
+        MG_TRY(halloc_t(H, &B.cfl, flags));
+        MG_CUDA_TRY(cudaMemsetAsync(B.cfl, 0, flags * sizeof(unsigned), s));
+        MG_TRY(halloc_t(H, &B.cgw, (size_t)NB_MAX / NB_TILE));
+        MG_CUDA_TRY(cudaMemsetAsync(B.cgw, 0, NB_MAX / NB_TILE * sizeof(unsigned long long), s));
     }
     MG_TRY(halloc_t(H, &B.oflags, (size_t)nbp));
     MG_TRY(halloc_t(H, &B.gates, (size_t)nbp));
@@ -301,6 +312,11 @@ mg_status bcoarse_proj(Handle& H, const float2* f, float2* x, int nb, Gate act, 
     cb.h2 = B.ch2;
     cb.ticket = B.ctk;
     cb.bar = B.cbar;
+    cb.t1 = B.ctw;
+    cb.t2 = B.ctw + cb_chunk_words(nb);
+    cb.flags = B.cfl;
+    cb.gword = B.cgw;
+    cb.epoch = B.cfl + cb_chunk_flags();
     cb.probe = B.probe;
     // the cycle kernel when its grid can be resident at once, else the step kernels
     const bool coop = !B.no_coop && cb_geometry_cycle(cb, (long)cb.Nx * cb.Nt, nb, fp16);
