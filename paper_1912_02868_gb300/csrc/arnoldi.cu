@@ -246,12 +246,14 @@ constexpr int FU_STEPS = 8;  // longest cycle of k_finish_update
 template <typename T>
 __global__ void __launch_bounds__(256) k_finish_update(C2<T>* __restrict__ x, C2<T>* __restrict__ r,
                                                        const C2<T>* __restrict__ V, long n, KState* ks, int accumulate) {
-    __shared__ double2 ds[FU_STEPS], rhos[FU_STEPS + 1];
+    __shared__ double2 Rs[FU_STEPS * (FU_STEPS + 1) / 2], ds[FU_STEPS], rhos[FU_STEPS + 1];
     __shared__ C2<T> dc[FU_STEPS], rc[FU_STEPS + 1];
     const int jj = ks->j;
     if (threadIdx.x < 32) {
         const int lane = threadIdx.x;
-        ksd::solve_upper<FU_STEPS>(ks->R, ks->g, ds, jj, blockIdx.x == 0 ? &ks->err : nullptr);
+        ksd::load_upper(Rs, ks->R, jj, lane, 32);
+        __syncwarp();
+        ksd::solve_upper(Rs, ks->g, ds, jj, blockIdx.x == 0 ? &ks->err : nullptr);
         double part = 0.0;
         if (lane <= jj) {
             double2 acc = ks->c[lane];

@@ -161,6 +161,12 @@ __global__ void __launch_bounds__(BT) k_bgram(double2* __restrict__ out, long os
     }
 }
 
+// Rows whose loads k_baxpy and k_bupdate keep in flight.  FP32 waits for memory: with one
+// row at a time the updates of a 256^2 solve of 64 right-hand sides took 65 ms, with five
+// and x and r of a cycle in one pass 40 ms.  FP64 is bound by its pipe and only loses warps
+// to the registers (17 ms with one row, 26 ms with five).
+template <typename T> constexpr int rows_ahead() { return sizeof(T) == 4 ? 5 : 1; }
+
 template <typename T>
 __global__ void __launch_bounds__(BT) k_baxpy(C2<T>* w, long wr, const C2<T>* __restrict__ V, long ldv, long vr,
                                               int nd, const int* ndd, long nds, const double2* __restrict__ coef,
@@ -168,6 +174,7 @@ __global__ void __launch_bounds__(BT) k_baxpy(C2<T>* w, long wr, const C2<T>* __
                                               C2<T>* partial, int max_chunks, unsigned* ticket, Gate g) {
     const int r = blockIdx.y;
     if (!gate_open(g, r)) return;
+    constexpr int BU = rows_ahead<T>();
     __shared__ C2<T> cf[RED_MAXD];
     __shared__ C2<T> sm[BT / 32];
     int cnt = nd + (ndd ? ndd[r * nds] : 0);
@@ -183,7 +190,14 @@ __global__ void __launch_bounds__(BT) k_baxpy(C2<T>* w, long wr, const C2<T>* __
     T tacc = 0;
     for (long e = (long)blockIdx.x * BT + threadIdx.x; e < n; e += stride) {
         C2<T> a = zero_first ? mk<T>(0, 0) : wv[e];
-        for (int i = 0; i < cnt; ++i) a = cfma(Vr[(long)i * ldv + e], cf[i], a);
+        for (int i = 0; i < cnt; i += BU) {  // BU rows' loads in flight (a row past the last repeats it)
+            C2<T> v[BU];
+#pragma unroll
+            for (int c = 0; c < BU; ++c) v[c] = Vr[(long)min(i + c, cnt - 1) * ldv + e];
+#pragma unroll
+            for (int c = 0; c < BU; ++c)
+                if (i + c < cnt) a = cfma(v[c], cf[i + c], a);
+        }
         wv[e] = a;
         if (norm2) tacc += a.x * a.x + a.y * a.y;
     }
@@ -201,6 +215,41 @@ __global__ void __launch_bounds__(BT) k_baxpy(C2<T>* w, long wr, const C2<T>* __
                 }
             }
         }
+    }
+}
+
+// A finished cycle of cnt[r cs] steps in one pass over its basis: x = V d (or x += V d) and,
+// unless r is null, r = V rho (cnt + 1 rows)
+template <typename T>
+__global__ void __launch_bounds__(BT) k_bupdate(C2<T>* x, long xr, C2<T>* rv, long rr, const C2<T>* __restrict__ V,
+                                                long ldv, long vr, const int* __restrict__ cnt, long cs,
+                                                const double2* __restrict__ d, const double2* __restrict__ rho, long ds,
+                                                int accumulate, long n, Gate g) {
+    const int r = blockIdx.y;
+    if (!gate_open(g, r)) return;
+    constexpr int BU = rows_ahead<T>();
+    __shared__ C2<T> cd[RED_MAXD], cr[RED_MAXD];
+    const int nd = min(cnt[r * cs], RED_MAXD - 1), rows = rv ? nd + 1 : nd;
+    for (int i = threadIdx.x; i < rows; i += BT) {
+        cd[i] = i < nd ? from_d2<T>(d[r * ds + i]) : mk<T>(0, 0);
+        cr[i] = rv ? from_d2<T>(rho[r * ds + i]) : mk<T>(0, 0);
+    }
+    __syncthreads();
+    const C2<T>* Vr = V + r * vr;
+    for (long e = (long)blockIdx.x * BT + threadIdx.x; e < n; e += (long)gridDim.x * BT) {
+        C2<T> a = accumulate ? x[r * xr + e] : mk<T>(0, 0), b = mk<T>(0, 0);
+        for (int i = 0; i < rows; i += BU) {
+            C2<T> v[BU];
+#pragma unroll
+            for (int c = 0; c < BU; ++c) v[c] = Vr[(long)min(i + c, rows - 1) * ldv + e];
+#pragma unroll
+            for (int c = 0; c < BU; ++c) {
+                if (i + c < nd) a = cfma(v[c], cd[i + c], a);
+                if (i + c < rows) b = cfma(v[c], cr[i + c], b);
+            }
+        }
+        x[r * xr + e] = a;
+        if (rv) rv[r * rr + e] = b;
     }
 }
 
@@ -255,13 +304,15 @@ __global__ void k_bconvert(C2<Tb>* y, long yr, const C2<Ta>* x, long xr, long n)
 }
 
 inline int chunks_for(long n, const BRed& red) {
-    long c = (n + BT * 4 - 1) / (BT * 4);
+    // an entry a thread: short vectors are bound by latency (with four, a 256^2 solve of 64
+    // right-hand sides took 1% longer)
+    long c = (n + BT - 1) / BT;
     if (c > red.max_chunks) c = red.max_chunks;
     if (c < 1) c = 1;
     return (int)c;
 }
 inline unsigned ew_chunks(long n) {
-    long c = (n + 1023) / 1024;
+    long c = (n + 255) / 256;
     if (c > 64) c = 64;
     if (c < 1) c = 1;
     return (unsigned)c;
@@ -493,6 +544,15 @@ void launch_baxpy(C2<T>* w, long wr, const C2<T>* V, long ldv, long vr, int nd, 
 }
 
 template <typename T>
+void launch_bupdate(C2<T>* x, long xr, C2<T>* r, long rr, const C2<T>* V, long ldv, long vr, const int* cnt, long cs,
+                    const double2* d, const double2* rho, long ds, bool accumulate, long n, int nb, Gate g,
+                    cudaStream_t s) {
+    const unsigned ch = (unsigned)std::max(1L, std::min((n + BT - 1) / BT, 64L));
+    k_bupdate<T><<<dim3(ch, nb), BT, 0, s>>>(x, xr, r, rr, V, ldv, vr, cnt, cs, d, rho, ds, accumulate ? 1 : 0, n, g);
+    count_launch();
+}
+
+template <typename T>
 void launch_bnorm2(double* out, long os, const C2<T>* v, long vr, long n, int nb, BRed red, Gate g, cudaStream_t s) {
     const int ch = chunks_for(n, red);
     k_bnorm2<T><<<dim3(ch, nb), BT, 0, s>>>(out, os, v, vr, n, reinterpret_cast<C2<T>*>(red.partial), red.max_chunks,
@@ -556,6 +616,8 @@ void launch_bstencil_mma(float2* Y, const float2* X, const float2* B, long vr, c
                                   long, long, int, BRed, Gate, cudaStream_t);                                      \
     template void launch_baxpy<T>(C2<T>*, long, const C2<T>*, long, long, int, const int*, long, const double2*,    \
                                   long, double, bool, long, int, double*, long, BRed, Gate, cudaStream_t);         \
+    template void launch_bupdate<T>(C2<T>*, long, C2<T>*, long, const C2<T>*, long, long, const int*, long,         \
+                                    const double2*, const double2*, long, bool, long, int, Gate, cudaStream_t);      \
     template void launch_bnorm2<T>(double*, long, const C2<T>*, long, long, int, BRed, Gate, cudaStream_t);         \
     template void launch_bscale<T>(C2<T>*, long, const C2<T>*, long, const double*, long, long, int, Gate,          \
                                    cudaStream_t);

@@ -27,6 +27,12 @@ template <typename T>
 void launch_baxpy(C2<T>* w, long wr, const C2<T>* V, long ldv, long vr, int nd, const int* ndd, long nds,
                   const double2* coef, long cs, double sign, bool zero_first, long n, int nb, double* norm2,
                   long n2s, BRed red, Gate g, cudaStream_t s);
+// x[r] = V[r] d[r] (or x[r] += V[r] d[r]) over cnt[r*cs] rows and, unless r is null,
+// r[r] = V[r] rho[r] over one more; d and rho at r*ds
+template <typename T>
+void launch_bupdate(C2<T>* x, long xr, C2<T>* r, long rr, const C2<T>* V, long ldv, long vr, const int* cnt, long cs,
+                    const double2* d, const double2* rho, long ds, bool accumulate, long n, int nb, Gate g,
+                    cudaStream_t s);
 template <typename T>
 void launch_bnorm2(double* out, long os, const C2<T>* v, long vr, long n, int nb, BRed red, Gate g, cudaStream_t s);
 // y[r] = x[r] * f[r*fs]

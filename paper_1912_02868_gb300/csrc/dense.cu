@@ -36,23 +36,46 @@ __global__ void k_bks_push(KState* ks, int jh) {
     ks_push_warp(ks + blockIdx.x, jh, S);
 }
 
+// A finished cycle's d = R^{-1} g and rho = c - H d by FIN_T threads: four threads a row of
+// H, which load their columns before the back substitution (one warp) starts, so that no
+// load follows it.
+constexpr int FIN_T = 256;
 __device__ void ks_finish_dev(KState* ks) {
-    const int jj = ks->j;
-    const int lane = threadIdx.x & 31;
-    solve_upper<KMAX>(ks->R, ks->g, ks->d, jj, &ks->err);
-    __syncwarp();
-    double part = 0.0;
-    for (int i = lane; i <= jj; i += 32) {
-        double2 acc = ks->c[i];
-#pragma unroll 8
-        for (int l = 0; l < jj; ++l) acc = csub(acc, cmul(ks->H[i + KLD * l], ks->d[l]));
-        ks->rho[i] = acc;
-        part += acc.x * acc.x + acc.y * acc.y;
-    }
-    for (int i = jj + 1 + lane; i < KLD; i += 32) ks->rho[i] = z0();
+    __shared__ double2 Rs[KMAX * (KMAX + 1) / 2], ds[KMAX];
+    __shared__ double part[FIN_T / 32];
+    const int jj = ks->j, tid = threadIdx.x, i = tid >> 2, q = tid & 3;
+    constexpr int HC = KMAX / 4;
+    static_assert(FIN_T / 4 >= KLD && KMAX % 4 == 0, "four threads a row");
+    load_upper(Rs, ks->R, jj, tid, FIN_T);
+    double2 h[HC];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-    if (lane == 0) ks->res = sqrt(part);
+    for (int c = 0; c < HC; ++c) {
+        const int l = q + 4 * c;
+        h[c] = i <= jj && l < jj ? ks->H[i + KLD * l] : z0();
+    }
+    double2 acc = i <= jj && q == 0 ? ks->c[i] : z0();
+    __syncthreads();
+    if (tid < 32) solve_upper(Rs, ks->g, ds, jj, &ks->err);
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < HC; ++c)
+        if (q + 4 * c < jj) acc = csub(acc, cmul(h[c], ds[q + 4 * c]));
+#pragma unroll
+    for (int o = 1; o <= 2; o <<= 1) {
+        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
+        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+    }
+    if (q == 0 && i < KLD) ks->rho[i] = i <= jj ? acc : z0();
+    if (tid < jj) ks->d[tid] = ds[tid];
+    double n2 = q == 0 && i <= jj ? acc.x * acc.x + acc.y * acc.y : 0.0;
+#pragma unroll
+    for (int o = 16; o >= 4; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+    if ((tid & 31) == 0) part[tid >> 5] = n2;
+    __syncthreads();
+    if (tid == 0) {
+        for (int w = 1; w < FIN_T / 32; ++w) n2 += part[w];
+        ks->res = sqrt(n2);
+    }
 }
 __global__ void k_ks_finish(KState* ks) { ks_finish_dev(ks); }
 __global__ void k_bks_finish(KState* ks) { ks_finish_dev(ks + blockIdx.x); }
@@ -122,13 +145,16 @@ __global__ void k_ks_load_dense(KState* ks, const double2* Hk, const double2* ck
 __global__ void k_proj_mats(const KState* pls, ProjMats* pm, int k) {
     __shared__ double2 g[KLD];
     __shared__ double2 ds[KMAX];
+    __shared__ double2 Rs[KMAX * (KMAX + 1) / 2];
     const int lane = threadIdx.x & 31, l = blockIdx.x;
     for (int i = lane; i < KLD; i += 32) g[i] = (i == l) ? make_double2(1.0, 0.0) : z0();
     __syncwarp();
     if (lane == 0)
         for (int t = 0; t < pls->nrot; ++t) rot_apply(pls->rc[t], pls->rs[t], g[pls->ra[t]], g[pls->rb[t]]);
     __syncwarp();
-    solve_upper<KMAX>(pls->R, g, ds, k, nullptr);
+    load_upper(Rs, pls->R, k, threadIdx.x, 32);
+    __syncwarp();
+    solve_upper(Rs, g, ds, k, nullptr);
     __syncwarp();
     for (int i = lane; i < k; i += 32) pm->M[i + k * l] = ds[i];
     for (int i = lane; i <= k; i += 32) {
@@ -563,7 +589,7 @@ void bks_push(KState* ks, int nb, int jh, cudaStream_t s) {
     count_launch();
 }
 void bks_finish(KState* ks, int nb, cudaStream_t s) {
-    k_bks_finish<<<nb, 32, 0, s>>>(ks);
+    k_bks_finish<<<nb, FIN_T, 0, s>>>(ks);
     count_launch();
 }
 void proj_mats(const KState* pls, ProjMats* pm, int k, cudaStream_t s) {
@@ -593,7 +619,7 @@ void ks_push(KState* ks, int jh, cudaStream_t s) {
     count_launch();
 }
 void ks_finish(KState* ks, cudaStream_t s) {
-    k_ks_finish<<<1, 32, 0, s>>>(ks);
+    k_ks_finish<<<1, FIN_T, 0, s>>>(ks);
     count_launch();
 }
 void ks_load_dense(KState* ks, const double2* Hk, const double2* ck, int k, double tol_abs, cudaStream_t s) {

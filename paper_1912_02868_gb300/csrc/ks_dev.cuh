@@ -173,18 +173,21 @@ __device__ inline void ks_push_warp(KState* ks, int jh, PushScratch& S) {
     __syncwarp();
     for (int i = lane; i < KLD; i += 32) ks->R[i + KLD * j] = col[i];
 }
-// Back substitution R d = g over the first jj <= MAXJ columns, by one warp: R is read
-// into shared memory at once, the lanes form the reciprocals of their pivots together
-// (a zero pivot gives d_i = 0 and *err = 2), and each column then costs a product, a
-// broadcast and a subtraction on the serial chain.  k_bks_finish for 64 right-hand
-// sides: 39 us with R and the divides on one thread, 24 us so.
-template <int MAXJ>
-__device__ inline void solve_upper(const double2* R, const double2* g, double2* d, int jj, int* err) {
-    __shared__ double2 Rs[MAXJ * (MAXJ + 1) / 2];  // column i: rows 0..i at i (i + 1) / 2
+// Columns 0..jj - 1 of the upper triangle R, column i's rows 0..i at i (i + 1) / 2, by nt
+// threads: several loads of a thread are in flight (a loop over columns waited for each:
+// 14 us of the 31 us k_bks_finish took)
+__device__ __forceinline__ void load_upper(double2* Rs, const double2* R, int jj, int tid, int nt) {
+#pragma unroll 4
+    for (int e = tid; e < jj * jj; e += nt) {
+        const int i = e / jj, r = e - i * jj;
+        if (r <= i) Rs[i * (i + 1) / 2 + r] = R[r + KLD * i];
+    }
+}
+// Back substitution R d = g over the first jj < 64 columns, by one warp: the lanes form the
+// reciprocals of their pivots together (a zero pivot gives d_i = 0 and *err = 2), and each
+// column then costs a product, a broadcast and a subtraction on the serial chain.
+__device__ inline void solve_upper(const double2* Rs, const double2* g, double2* d, int jj, int* err) {
     const int lane = threadIdx.x & 31;
-    for (int i = 0; i < jj; ++i)
-        for (int r = lane; r <= i; r += 32) Rs[i * (i + 1) / 2 + r] = R[r + KLD * i];
-    __syncwarp();
     double2 acc[2], inv[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {

@@ -267,11 +267,8 @@ void bsmoother(Handle& H, int l, const float2* f, float2* x, bool accumulate, fl
         barnoldi_step<float>(B, [&](float2* w, const float2* in, Gate g) { bapply(H, l, w, in, nullptr, nb, g, s); },
                              W.sV, n, nb, W.ks, jh, s);
     bks_finish(W.ks, nb, s);
-    launch_baxpy<float>(x, n, W.sV, row, n, 0, MG_DEVF(W.ks, int, j), KS_INTS, MG_DEVF(W.ks, double2, d), KS_CPLX,
-                        1.0, !accumulate, n, nb, nullptr, 0, B.red, act, s);
-    if (r_out)
-        launch_baxpy<float>(r_out, n, W.sV, row, n, 1, MG_DEVF(W.ks, int, j), KS_INTS, MG_DEVF(W.ks, double2, rho),
-                            KS_CPLX, 1.0, true, n, nb, nullptr, 0, B.red, act, s);
+    launch_bupdate<float>(x, n, r_out, n, W.sV, row, n, MG_DEVF(W.ks, int, j), KS_INTS, MG_DEVF(W.ks, double2, d),
+                          MG_DEVF(W.ks, double2, rho), KS_CPLX, accumulate, n, nb, act, s);
 }
 
 // GMRES-Proj(m,k) on the coarsest grid for every right-hand side with an open
@@ -342,10 +339,8 @@ mg_status bcoarse_proj(Handle& H, const float2* f, float2* x, int nb, Gate act, 
         else
             for (int jh = 0; jh < ms; ++jh) launch_cb_step(cb, jh, fp16, cs);
         bks_finish(B.cks, nb, cs);
-        launch_baxpy<float>(x, n, B.cV, row, n, 0, MG_DEVF(B.cks, int, j), KS_INTS, MG_DEVF(B.cks, double2, d),
-                            KS_CPLX, 1.0, false, n, nb, nullptr, 0, B.red, ca, cs);
-        launch_baxpy<float>(B.cr, n, B.cV, row, n, 1, MG_DEVF(B.cks, int, j), KS_INTS, MG_DEVF(B.cks, double2, rho),
-                            KS_CPLX, 1.0, true, n, nb, nullptr, 0, B.red, ca, cs);
+        launch_bupdate<float>(x, n, B.cr, n, B.cV, row, n, MG_DEVF(B.cks, int, j), KS_INTS,
+                              MG_DEVF(B.cks, double2, d), MG_DEVF(B.cks, double2, rho), KS_CPLX, true, n, nb, ca, cs);
         k_coarse_cycle_end<<<1, 64, 0, cs>>>(B.cact, B.citers, B.cks, nb, B.ccycles, H.p.proj_max_cycles, B.count);
         count_launch();
     };
