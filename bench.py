@@ -668,7 +668,7 @@ def run_native(args):
     roofline = {"bound": "hbm", "achieved": c_ach, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                 "frac": c_ach / peaks["hbm_gbs"],
                 "traffic": profile_of("coarse_proj_f32_256.json").get("dram_bytes_per_launch"),
-                "kernel": "k_coarse_proj<float> (whole coarse GMRES-Proj solve, 16^2 x 24, FP16 operator"
+                "kernel": "k_coarse_tc (whole coarse GMRES-Proj solve, 16^2 x 24, FP16 operator"
                           + (" applied on tensor cores" if args.coarse_mma else "") + ", cluster of 16 CTAs)",
                 "bytes_per_launch": c_bytes, "steps_per_launch": steps_per_launch,
                 "us_per_step": 1e6 * c_avg / max(steps_per_launch, 1), "avg_launch_us": c_avg * 1e6,
@@ -676,17 +676,18 @@ def run_native(args):
                 "note": "latency-bound: each Krylov step is two DSMEM reductions and a neighbour exchange, "
                         "counted on mbarriers; the stencil operand (5.9 MB) is L2-resident, so HBM is not the "
                         "binding limit"}
-    # second bound: per Arnoldi step each of the 16 CTAs reads its two L2-streamed
-    # FP16 operator directions (16 sites x 2 x 576 x 4 B) from L2, and from shared
-    # memory the three held directions plus the basis rows of the two CGS2 passes
+    # second bound, per Arnoldi step and CTA of the 16.  Tensor-core apply: the operator
+    # stays on chip, 6144 B a site in shared memory (the rest in registers).  FMA apply:
+    # two FP16 operator directions (16 sites x 2 x 576 x 4 B) from L2, three from shared
+    # memory.  Both: the basis rows of the two CGS2 passes from shared memory
     # (2 x (ms + 1) / 2 rows of 16 x 24 complex64 on average over a cycle)
     l2_total = l2_copy_rate(torch, dev)
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
     l2_sm = l2_total / sms
     smem_sm = 128 * 2.07  # GB/s per SM: 128 B per cycle at the maximum SM clock (nominal)
     ms_c = max(H_DR_M - 10, 1)
-    l2_b = 16 * 2 * 576 * 4
-    sm_b = 16 * 3 * 576 * 4 + (ms_c + 1) * 16 * 24 * 8
+    l2_b = 0 if args.coarse_mma else 16 * 2 * 576 * 4
+    sm_b = (16 * 6144 if args.coarse_mma else 16 * 3 * 576 * 4) + (ms_c + 1) * 16 * 24 * 8
     t_floor = max(l2_b / (l2_sm * 1e9), sm_b / (smem_sm * 1e9))
     roofline["second_bound"] = {
         "what": "per-SM L2 and shared-memory rates; step floor = max(L2 bytes / L2 rate, SMEM bytes / SMEM rate)",
@@ -793,12 +794,12 @@ def run_native(args):
                                   "frac": ach / peaks["hbm_gbs"],
                                   "traffic": profile_of("cb_cycle_bf16_256_64rhs.json").get("dram_bytes_per_step"),
                                   "traffic_unit": "bytes per lockstep step",
-                                  "kernel": "k_cb_cycle<bf16> (batched coarse GMRES-Proj, 16^2 x 24, 64 RHS, "
+                                  "kernel": "k_cb_chunk<bf16> (batched coarse GMRES-Proj, 16^2 x 24, 64 RHS, "
                                             "one cooperative kernel per GMRES cycle)",
                                   "us_per_step": 1e3 * cms / steps, "steps": steps, "bytes_per_step": step_bytes,
                                   "ms": cms, "peak_source": peak_kind,
-                                  "note": "the Krylov bases of the 64 right-hand sides (65 MB) stay in L2; each "
-                                          "step is three tile barriers apart"}
+                                  "note": "the Krylov bases of the 64 right-hand sides (65 MB) stay in L2 and shared "
+                                          "memory; each step has two exchanges of sums and one row flag"}
             h.close()
         batching["what"] = ("64 right-hand sides of one 256^2 configuration in one mg_solve: lockstep block "
                             "solve with the 24x24 block products of the intermediate and coarsest grids on tensor "
