@@ -174,8 +174,7 @@ __device__ inline void ks_push_warp(KState* ks, int jh, PushScratch& S) {
     for (int i = lane; i < KLD; i += 32) ks->R[i + KLD * j] = col[i];
 }
 // Columns 0..jj - 1 of the upper triangle R, column i's rows 0..i at i (i + 1) / 2, by nt
-// threads: several loads of a thread are in flight (a loop over columns waited for each:
-// 14 us of the 31 us k_bks_finish took)
+// threads: several loads of a thread are in flight (a loop over columns waited for each)
 __device__ __forceinline__ void load_upper(double2* Rs, const double2* R, int jj, int tid, int nt) {
 #pragma unroll 4
     for (int e = tid; e < jj * jj; e += nt) {
