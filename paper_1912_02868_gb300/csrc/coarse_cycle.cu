@@ -19,9 +19,10 @@
 //    is one store and one load, without barrier, fence or counter.  The new basis row is
 //    published by one release flag a CTA; the stop decisions by one tagged word a tile,
 //    made from one FP64 dot product while the rotations run on a warp nobody waits for.
-// A cycle of 20 steps, 256^2 x 64: 788 -> 498 us (24.9 us a step); the whole solve 511 ->
-// 418 ms.  Still latencies: apply 7 us (an L2 round is 0.6 us), the two passes over the
-// rows 3.4 and 6.7 us, their exchanges 3 us each, the update 2.8 us.
+// A cycle of 20 steps, 256^2 x 64, alone and cold: 788 -> 572 us (28.6 us a step); with the
+// projection and finish around it 48.4 -> 34.5 us a step; the whole solve 511 -> 418 ms.
+// Still latencies (L2 at 16% of its rate): apply 7 us (an L2 round is 0.6 us), the two
+// passes over the rows 3.4 and 6.7 us, their exchanges 3 us each, the update 2.8 us.
 //
 // Reuse of the exchange words: a CTA writes partials of step j + 1 only after every
 // CTA of the tile has raised its flag of step j, which it does after reading all
