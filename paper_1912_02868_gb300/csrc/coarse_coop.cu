@@ -770,18 +770,20 @@ __global__ void __maxnreg__(128) k_coarse_proj(CoopArgs<T> a) {
         return ms;
     };
     // Row updates w - V h of few rows in FP64 (one site a CTA): PS adjacent lanes share a
-    // row's products, so that three schedulers work instead of one
+    // row's products, so that three schedulers work instead of one.  The lanes of a row run
+    // different numbers of products; the full mask brings the warp together again (a site's
+    // NDOF * PS threads are whole warps).
     constexpr int PS = 4;
+    static_assert(NDOF * PS % 32 == 0, "the threads of a site's row updates are whole warps");
     const bool split_rows = std::is_same<T, double>::value && flow && a.lsw && nrows * PS <= 96 && nwr * 32 >= 96;
     auto accum_split = [&](const Z* w, const Z* h, int cnt) {
         const int e = tid / PS, q0 = tid % PS;
         Z acc = q0 == 0 ? w[e] : mk<T>(0, 0);
         for (int i = q0; i < cnt; i += PS) acc = cfms_<T>(Vl[(long)i * ldv + e], h[i], acc);
-        const unsigned m = __activemask();
 #pragma unroll
         for (int o = PS / 2; o > 0; o >>= 1) {
-            acc.x += __shfl_xor_sync(m, acc.x, o);
-            acc.y += __shfl_xor_sync(m, acc.y, o);
+            acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
+            acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
         }
         return acc;
     };
@@ -921,14 +923,15 @@ __global__ void __maxnreg__(128) k_coarse_proj(CoopArgs<T> a) {
                         Psum[tid] = acc;
                     }
                     if (!ls_warp) row_warps_sync(nwr * 32);
-                    // each real component by itself; with many groups, four lanes a component
+                    // each real component by itself; with many groups, four lanes a component (then
+                    // a CTA has one site or none: its 8 NDOF threads are whole warps)
                     const T* ps = reinterpret_cast<const T*>(Psum);
                     const int ql = a.ks >= 12 ? 4 : 1;
                     if (tid < 2 * nrows * ql) {
                         const int c = tid / ql, q0 = tid - c * ql;
                         T acc = 0;
                         for (int q = q0; q < a.ks; q += ql) acc += ps[(long)q * 2 * nrows + c];
-                        for (int o = ql >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(__activemask(), acc, o);
+                        for (int o = ql >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
                         if (q0 == 0) reinterpret_cast<T*>(wl)[c] = acc;
                     }
                 } else {
