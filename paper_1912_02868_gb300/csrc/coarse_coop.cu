@@ -996,12 +996,11 @@ __global__ void __maxnreg__(128) k_coarse_proj(CoopArgs<T> a) {
                 for (int o = 16; o > 0; o >>= 1) h2n += __shfl_xor_sync(0xffffffffu, h2n, o);
                 const T hh = fmax((T)S.red[j + 1].x - h2n, T(0));
                 if constexpr (std::is_same<T, double>::value) {
-                    // one reciprocal square root and a correction step instead of the square
-                    // root and the division one after the other
+                    // the rows need the reciprocal and the least squares the root: each warp forms
+                    // its own, not a root and a division one after the other
                     if (hh > T(0)) {
-                        sc = rsqrt(hh);
-                        hn = hh * sc;
-                        hn = fma(fma(-hn, hn, hh), T(0.5) * sc, hn);
+                        if (!ls_warp) sc = rsqrt(hh);
+                        if (a.lsw ? ls_warp : tid < 32) hn = sqrt(hh);
                     }
                 } else {
                     hn = sqrt(hh);

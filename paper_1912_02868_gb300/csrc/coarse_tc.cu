@@ -83,7 +83,7 @@ struct alignas(16) TcSmem {
         float rc[MSMAX];                // rotations
         float2 rs[MSMAX], g[MSMAX + 1], d[MSMAX];
     } st;
-    double tol_abs;
+    double tol2;  // square of the tolerance on ||r||
     float sc, beta;
     int ctl[4];
     unsigned long long mb[4];  // inbox 0, inbox 1, staged rows; [3]: the probe's, which nothing completes
@@ -254,25 +254,6 @@ __device__ __forceinline__ void tc_gram(const float2* X, long ldx, int nd, const
                       __float_as_uint(v.y), __float_as_uint(ox), __float_as_uint(oy), cluster_addr(bar, lane));
     }
 }
-
-// sqrt(x) and 1 / sqrt(x) from the hardware estimate and one Newton step each, for
-// x >= 0 (x = 0: 0 and 0): within a rounding of the IEEE sequences, without their
-// slow-path calls, which cost registers in the step loop
-__device__ __forceinline__ float2 sqrt_rsqrt(float x) {
-    if (!(x > 0.f)) return make_float2(0.f, 0.f);
-    const float r0 = rsqrtf(x), s0 = x * r0;
-    const float r = fmaf(0.5f * r0, fmaf(-s0, r0, 1.f), r0);
-    return make_float2(fmaf(fmaf(-s0, s0, x), 0.5f * r0, s0), r);
-}
-// the same in FP64 (estimate in FP32, two steps)
-__device__ __forceinline__ double2 sqrt_rsqrt_d(float x) {
-    if (!(x > 0.f)) return make_double2(0.0, 0.0);
-    double y = (double)rsqrtf(x);
-    y = y * (1.5 - 0.5 * (double)x * y * y);
-    y = y * (1.5 - 0.5 * (double)x * y * y);
-    return make_double2((double)x * y, y);
-}
-
 
 // red[i] = sum over the inbox rows of column i, i < nd (and column nd into *nrm), half
 // a warp a column, in one fixed tree (at most 16 rows): every CTA gets the same bits.
@@ -604,7 +585,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1) k_coarse_tc(const __
             st.rc[jc] = cc;
             st.rs[jc] = ss;
             st.g[jc] = gj;
-            S.ctl[0] = ((double)(g_ls.x * g_ls.x + g_ls.y * g_ls.y) <= S.tol_abs * S.tol_abs) ? 1 : 0;
+            S.ctl[0] = ((double)(g_ls.x * g_ls.x + g_ls.y * g_ls.y) <= S.tol2) ? 1 : 0;
             S.ctl[1] = (hnv == 0.f) ? 1 : 0;
         }
     };
@@ -632,7 +613,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1) k_coarse_tc(const __
         // S.ctl[0]: the last cycle converged (the same in every CTA that has not faulted)
         if (anyf | S.ctl[0] | (cycles >= a.max_cycles)) break;
         if (cycles == 0 && tid == 0)  // r = f: the tolerance is relative to ||f||
-            S.tol_abs = a.tol * sqrt_rsqrt_d(S.nrm[0]).x;
+            S.tol2 = a.tol * a.tol * (double)fmaxf(S.nrm[0], 0.f);
         {
             const float2* Mp = reinterpret_cast<const float2*>(smem_raw + g.o_m);
             const float2* Np = Mp + k * (k + 1);
@@ -666,15 +647,15 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1) k_coarse_tc(const __
         }
         __syncthreads();
         exchange(1, V, ldv, 0, V);
-        // beta = ||r||, the stop test, and the start of the cycle
+        // beta = ||r||, the stop test (on squares), and the start of the cycle; the scale, an
+        // FP64 reciprocal root rounded to FP32, on another warp
+        const float b2 = fmaxf(S.nrm[1], 0.f);
         if (tid == 0) {
-            const double2 bs = sqrt_rsqrt_d(S.nrm[1]);
-            const double beta = bs.x;
-            S.ctl[0] = (beta <= S.tol_abs || beta == 0.0) ? 1 : 0;
+            S.ctl[0] = ((double)b2 <= S.tol2 || b2 == 0.f) ? 1 : 0;
             S.ctl[1] = 0;
-            S.sc = (float)bs.y;
-            S.beta = (float)beta;
+            S.beta = sqrtf(b2);
         }
+        if (tid == 32) S.sc = b2 > 0.f ? (float)rsqrt((double)b2) : 0.f;
         __syncthreads();
         if (S.ctl[0]) continue;  // converged: leave at the next round's barrier
         // ---- one GMRES(ms) cycle from r ----
@@ -757,7 +738,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1) k_coarse_tc(const __
                 }
             }
             // h_{j+1,j} = ||w - V h2|| = sqrt(n2 - |h2|^2) (V orthonormal), the same bits in
-            // every thread; then v_{j+1} = (w - V h2) / h_{j+1,j}
+            // every thread; then v_{j+1} = (w - V h2) / h_{j+1,j}.
             float h2n = 0.f;
             if (lane <= j) {
                 const float4 h = S.red[1][lane];
@@ -765,19 +746,19 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1) k_coarse_tc(const __
             }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) h2n += __shfl_xor_sync(0xffffffffu, h2n, o);
-            const float2 hr = sqrt_rsqrt(S.nrm[1] - h2n);  // h_{j+1,j} and its reciprocal
+            const float hn = sqrtf(fmaxf(S.nrm[1] - h2n, 0.f)), inv = hn > 0.f ? 1.f / hn : 0.f;
             TC_STAMP(10);
             arm(2, S.nremote * XW * 4);
             if (warp * 32 < nrows) {
                 float2 v = make_float2(0.f, 0.f);
                 if (row_on) {
-                    v = cscale(csub(wl[tid], tc_combine<false>(V + tid, ldv, S.red[1], j + 1)), hr.y);
+                    v = cscale(csub(wl[tid], tc_combine<false>(V + tid, ldv, S.red[1], j + 1)), inv);
                     wl[tid] = v;
                 }
                 TC_STAMP(11);
                 stage(v);
             }
-            if (warp == NW - 1) ls_update(j, hr.x);
+            if (warp == NW - 1) ls_update(j, hn);
             TC_STAMP(5);
 #ifdef CP_PHASE_CLOCKS
             ++clk_steps;
