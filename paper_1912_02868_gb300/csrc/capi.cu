@@ -59,7 +59,7 @@ mg_status clear_coarse_exchange(Handle& H, cudaStream_t s) {
     if (!H.cpart) return MG_OK;
     MG_CUDA_TRY(cudaMemsetAsync(H.cpart, 0, (size_t)2 * H.cpart_ctas * PSTR * sizeof(double2), s));
     MG_CUDA_TRY(cudaMemsetAsync(H.crows, 0, (size_t)2 * H.L64[2].n * sizeof(double2), s));
-    MG_CUDA_TRY(cudaMemsetAsync(H.cepoch, 0, sizeof(unsigned), s));
+    MG_CUDA_TRY(cudaMemsetAsync(H.cepoch, 0, 2 * sizeof(unsigned), s));
     return MG_OK;
 }
 
@@ -205,7 +205,7 @@ mg_status alloc_workspaces(Handle& H, cudaStream_t s, bool owner) {
         H.cpart_ctas = sm_count();
         MG_TRY(halloc_t(H, &H.cpart, (size_t)2 * H.cpart_ctas * PSTR));
         MG_TRY(halloc_t(H, &H.crows, (size_t)2 * n2));
-        MG_TRY(halloc_t(H, &H.cepoch, 1));
+        MG_TRY(halloc_t(H, &H.cepoch, 2));
         MG_TRY(clear_coarse_exchange(H, s));
     }
     MG_TRY(halloc_t(H, &H.cstats, 1));

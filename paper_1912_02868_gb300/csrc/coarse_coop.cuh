@@ -33,7 +33,8 @@ struct CoopArgs {
     double tol;        // stop when ||r|| <= tol ||f||
     int max_cycles;
     // exchange buffers of the grid form of coarse_tc.cu (null: not allocated): tagged
-    // partial sums (2 x PSTR x part_ctas), tagged rows (2 x n) and the launch's tag base
+    // partial sums (2 x PSTR x part_ctas), tagged rows (2 x n), and the launch's tag base with
+    // a word that nothing writes (the probe's)
     double2* part;
     int part_ctas;
     double2* rows;
@@ -49,8 +50,8 @@ struct CoopArgs {
     int flow;          // 1: push mode exchanges each step's values by st.async into byte-counted
                        // barriers instead of cluster barriers (set by the launcher)
     long spin;         // try_wait rounds before a dataflow wait gives up (0: the default, 2^20)
-    int probe;         // 1 (tests): before the first cycle every row thread waits, bounded by
-                       // `spin`, on a barrier that nothing completes, so the give-up path runs
+    int probe;         // 1 (tests): before the first cycle every CTA waits, bounded by `spin`, on a
+                       // barrier that nothing completes, so the give-up path runs (dataflow forms)
     int mma;           // 1: the apply runs on tensor cores where it can (coarse_tc.cu: FP32 vectors,
                        // at most 16 sites a CTA, CGS2): FP16 operator times the vector split into
                        // two FP16 parts, FP32 accumulation

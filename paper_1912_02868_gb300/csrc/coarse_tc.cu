@@ -64,7 +64,7 @@ struct TcShape {
     // byte offsets in dynamic shared memory
     int o_inbox, o_x, o_v, o_m, o_op, o_sol, o_w;
     // GRID: tagged partial sums [2][PSTR][CTAs], tagged rows [2][sites x 24], and the tag
-    // base of this launch (advanced at its end)
+    // base of this launch (advanced at its end) with a word that nothing writes (the probe's)
     ulonglong2 *part, *rows;
     unsigned* epoch;
 };
@@ -461,7 +461,19 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1) k_coarse_tc(const __
         V[tid] = a.f[(long)s0 * NDOF + tid];
     }
     __syncthreads();
-    if (!GRID && a.probe && !S.fault && !mbar_wait(&S.mb[3], 0u, a.spin > 0 ? a.spin : FLOW_SPIN)) S.fault = 1;
+    if (a.probe) {  // test probe: a wait that nothing ends gives up
+        const long spin = a.spin > 0 ? a.spin : FLOW_SPIN;
+        if constexpr (GRID) {
+            if (tid == 0) {
+                long it = 0;
+                while (it < spin && __ldcg(g.epoch + 1) == 0u) ++it;
+                if (it == spin) S.fault = 1;
+            }
+        } else if (!S.fault && !mbar_wait(&S.mb[3], 0u, spin)) {
+            S.fault = 1;
+        }
+        __syncthreads();
+    }
     // a new basis row: an even row stages itself and its odd partner, in the own
     // site's slot and in those of the neighbouring CTAs that read it
     auto stage = [&](float2 v) {

@@ -154,7 +154,7 @@ struct Handle {
     KState* pls = nullptr;    // factored H_k of the deflation space
     ProjMats* pmat = nullptr; // its projection matrices
     // exchange buffers of the coarse solve over the whole GPU (grids of more than one
-    // cluster's sites): tagged partial sums, tagged rows, tag base
+    // cluster's sites): tagged partial sums, tagged rows, tag base (and the probe's word)
     double2* cpart = nullptr;
     int cpart_ctas = 0;
     double2* crows = nullptr;

@@ -5,6 +5,8 @@ cluster (64^2) and over the whole GPU (272 x 256: more than 256 coarse sites).
   and is zero at entries of 1e-30 and at zero): the solve ends with the projection onto the
   deflation space, as the general kernel (coarse_mma = 0) does, to the 1e-4 that both keep
   against the oracle.
+* A bounded wait that gives up (the probe: nothing ends it) makes the call return MG_ETIMEOUT
+  with every CTA counted, and the next solve is bitwise the one before the probe.
 """
 import numpy as np
 import pytest
@@ -56,3 +58,21 @@ def test_norms_beyond_fp32(mgmod, Lx, Lt):
         (it1, conv1, x1), (it0, conv0, x0) = got[1, scale], got[0, scale]
         assert (it1, conv1) == (it0, conv0) == (0, True)
         assert np.isfinite(x1).all() and rel2(x1, x0) <= 1e-4
+
+
+@pytest.mark.parametrize("Lx,Lt", SIZES)
+def test_probe_gives_up(mgmod, Lx, Lt):
+    import torch
+    g = _handle(mgmod, Lx, Lt)
+    try:
+        b = _rhs(Lx, Lt)
+        x, y, z = (torch.zeros_like(b) for _ in range(3))
+        _, it, conv, info = mgmod.mg_coarse_solve(g, b, x, 1e-5, mgmod.MG_F32)
+        assert conv[0] and info["tensor_apply"] == 1 and info["timeouts"] == 0
+        st, _, _, info = mgmod.mg_coarse_solve(g, b, y, 1e-5, mgmod.MG_F32, flags=mgmod.MG_COARSE_PROBE_TIMEOUT,
+                                               spin=64, allow=(mgmod.MG_OK, mgmod.MG_ETIMEOUT))
+        assert st == mgmod.MG_ETIMEOUT and info["timeouts"] == info["ctas"] >= 16
+        _, it2, conv2, info = mgmod.mg_coarse_solve(g, b, z, 1e-5, mgmod.MG_F32)
+        assert it2 == it and conv2[0] and info["timeouts"] == 0 and torch.equal(x, z)
+    finally:
+        g.close()
