@@ -55,11 +55,22 @@ mg_status halloc(Handle& H, void** p, size_t bytes) {
     return MG_OK;
 }
 
-mg_status clear_coarse_exchange(Handle& H, cudaStream_t s) {
-    if (!H.cpart) return MG_OK;
-    MG_CUDA_TRY(cudaMemsetAsync(H.cpart, 0, (size_t)2 * H.cpart_ctas * PSTR * sizeof(double2), s));
-    MG_CUDA_TRY(cudaMemsetAsync(H.crows, 0, (size_t)2 * H.L64[2].n * sizeof(double2), s));
-    MG_CUDA_TRY(cudaMemsetAsync(H.cepoch, 0, 2 * sizeof(unsigned), s));
+mg_status begin_coarse(Handle& H, cudaStream_t s) {
+    if (H.cpart && H.cdirty) {
+        MG_CUDA_TRY(cudaMemsetAsync(H.cpart, 0, (size_t)2 * H.cpart_ctas * PSTR * sizeof(double2), s));
+        MG_CUDA_TRY(cudaMemsetAsync(H.crows, 0, (size_t)2 * H.L64[2].n * sizeof(double2), s));
+        MG_CUDA_TRY(cudaMemsetAsync(H.cepoch, 0, 2 * sizeof(unsigned), s));
+    }
+    H.cdirty = true;
+    MG_CUDA_TRY(cudaMemsetAsync(H.cstats, 0, sizeof(CoopStats), s));
+    return MG_OK;
+}
+
+mg_status end_coarse(Handle& H, cudaStream_t s, CoopStats* cs) {
+    MG_CUDA_TRY(cudaMemcpyAsync(H.pinned, H.cstats, sizeof(CoopStats), cudaMemcpyDeviceToHost, s));
+    MG_CUDA_TRY(cudaStreamSynchronize(s));
+    std::memcpy(cs, H.pinned, sizeof *cs);
+    H.cdirty = cs->timeouts != 0;
     return MG_OK;
 }
 
@@ -206,7 +217,6 @@ mg_status alloc_workspaces(Handle& H, cudaStream_t s, bool owner) {
         MG_TRY(halloc_t(H, &H.cpart, (size_t)2 * H.cpart_ctas * PSTR));
         MG_TRY(halloc_t(H, &H.crows, (size_t)2 * n2));
         MG_TRY(halloc_t(H, &H.cepoch, 2));
-        MG_TRY(clear_coarse_exchange(H, s));
     }
     MG_TRY(halloc_t(H, &H.cstats, 1));
     if (p.partial_tol > 0.0) {
@@ -243,8 +253,7 @@ mg_status alloc_workspaces(Handle& H, cudaStream_t s, bool owner) {
 mg_status solve_rhs_pairs(Handle& A, Handle& Bh, const double2* B, double2* X, int first, int nrhs, int p0, int step,
                           double tol, cudaStream_t s, int* iters, double* relres) {
     const long n0 = A.L64[0].n;
-    MG_CUDA_TRY(cudaMemsetAsync(A.cstats, 0, sizeof(CoopStats), s));
-    MG_CUDA_TRY(cudaMemsetAsync(Bh.cstats, 0, sizeof(CoopStats), s));
+    for (Handle* Hp : {&A, &Bh}) MG_TRY(begin_coarse(*Hp, s));
     mg_status result = MG_OK;
     const int npairs = (nrhs - first + 1) / 2;
     for (int p = p0; p < npairs; p += step) {
@@ -273,18 +282,15 @@ mg_status solve_rhs_pairs(Handle& A, Handle& Bh, const double2* B, double2* X, i
             if (!conv[q]) result = MG_ENOTCONV;
         }
     }
+    long long timeouts = 0;
     for (Handle* Hp : {&A, &Bh}) {
         CoopStats cs{};
-        MG_CUDA_TRY(cudaMemcpyAsync(Hp->pinned, Hp->cstats, sizeof(CoopStats), cudaMemcpyDeviceToHost, s));
-        MG_CUDA_TRY(cudaStreamSynchronize(s));
-        std::memcpy(&cs, Hp->pinned, sizeof cs);
+        MG_TRY(end_coarse(*Hp, s, &cs));
         Hp->st.coarse_iters += cs.iters;
         Hp->st.mvps[2] += cs.iters;
-        if (cs.timeouts) {
-            MG_TRY(clear_coarse_exchange(*Hp, s));
-            return set_error("coarse solve: a bounded wait of the dataflow exchange gave up"), MG_ETIMEOUT;
-        }
+        timeouts += cs.timeouts;
     }
+    if (timeouts) return set_error("coarse solve: a bounded wait of the dataflow exchange gave up"), MG_ETIMEOUT;
     return result;
 }
 
@@ -299,7 +305,7 @@ mg_status solve_rhs(Handle& H, const double2* B, double2* X, bool bdev, bool xde
         const int k = H.p.method == MG_METHOD_FINE_DEFLATION ? H.fine_k : H.defl_k;
         if (needs && k == 0) return set_error("a solve context cannot build the deflation space"), MG_EINVAL;
     }
-    MG_CUDA_TRY(cudaMemsetAsync(H.cstats, 0, sizeof(CoopStats), s));
+    MG_TRY(begin_coarse(H, s));
     mg_status result = MG_OK;
     for (int i = i0; i < i1; i += step) {
         const double2* bi = B + (long)i * n0;
@@ -326,15 +332,10 @@ mg_status solve_rhs(Handle& H, const double2* B, double2* X, bool bdev, bool xde
         if (!conv) result = MG_ENOTCONV;
     }
     CoopStats cs{};
-    MG_CUDA_TRY(cudaMemcpyAsync(H.pinned, H.cstats, sizeof(CoopStats), cudaMemcpyDeviceToHost, s));
-    MG_CUDA_TRY(cudaStreamSynchronize(s));
-    std::memcpy(&cs, H.pinned, sizeof cs);
+    MG_TRY(end_coarse(H, s, &cs));
     H.st.coarse_iters += cs.iters;
     H.st.mvps[2] += cs.iters;
-    if (cs.timeouts) {
-        MG_TRY(clear_coarse_exchange(H, s));
-        return set_error("coarse solve: a bounded wait of the dataflow exchange gave up"), MG_ETIMEOUT;
-    }
+    if (cs.timeouts) return set_error("coarse solve: a bounded wait of the dataflow exchange gave up"), MG_ETIMEOUT;
     return result;
 }
 

@@ -129,7 +129,7 @@ mg_status mg_coarse_solve(mg_handle h, int precision, int nrhs, const void* b, v
         HH[1] = &H.contexts[0]->h;
         HH[1]->defl_k = H.defl_k;
     }
-    for (int r = 0; r < nrhs; ++r) MG_CUDA_TRY(cudaMemsetAsync(HH[r]->cstats, 0, sizeof(CoopStats), s));
+    for (int r = 0; r < nrhs; ++r) MG_TRY(begin_coarse(*HH[r], s));
     if (precision == MG_F64) {
         CoopArgs<double> a = coarse_args<double>(H, static_cast<const double2*>(b), static_cast<double2*>(x), H.c64.r,
                                                  H.c64.V, H.cpart, H.cpart_ctas, H.cstats, tol);
@@ -159,9 +159,7 @@ mg_status mg_coarse_solve(mg_handle h, int precision, int nrhs, const void* b, v
     long long timeouts = 0;
     CoopStats cs[2]{};
     for (int r = 0; r < nrhs; ++r) {
-        MG_CUDA_TRY(cudaMemcpyAsync(H.pinned, HH[r]->cstats, sizeof(CoopStats), cudaMemcpyDeviceToHost, s));
-        MG_CUDA_TRY(cudaStreamSynchronize(s));
-        std::memcpy(&cs[r], H.pinned, sizeof(CoopStats));
+        MG_TRY(end_coarse(*HH[r], s, &cs[r]));
         if (iters) iters[r] = cs[r].iters;
         if (converged) converged[r] = cs[r].unconverged == 0 ? 1 : 0;
         timeouts += cs[r].timeouts;
@@ -178,8 +176,6 @@ mg_status mg_coarse_solve(mg_handle h, int precision, int nrhs, const void* b, v
         info->cycles = cs[0].cycles;
         info->timeouts = timeouts;
     }
-    if (timeouts)
-        for (int r = 0; r < nrhs; ++r) MG_TRY(clear_coarse_exchange(*HH[r], s));
     if (timeouts) return set_error("coarse solve: a bounded wait of the dataflow exchange gave up"), MG_ETIMEOUT;
     return MG_OK;
 }

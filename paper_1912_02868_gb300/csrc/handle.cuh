@@ -159,6 +159,7 @@ struct Handle {
     int cpart_ctas = 0;
     double2* crows = nullptr;
     unsigned* cepoch = nullptr;
+    bool cdirty = true;       // they may hold anything (begin_coarse clears them)
     CoopStats* cstats = nullptr;
     // fine-grid deflation arm (method MG_METHOD_FINE_DEFLATION), FP64
     double2* fdV = nullptr;   // (m+1) x n0
@@ -199,9 +200,12 @@ template <> inline PartialWS<float>& Handle::partial<float>() { return p32; }
 
 // allocation owned by the handle
 mg_status halloc(Handle& H, void** p, size_t bytes);
-// clears the exchange buffers of the grid-wide coarse solve (at allocation, and after a
-// solve in which a wait gave up: its CTAs' tags may have run apart)
-mg_status clear_coarse_exchange(Handle& H, cudaStream_t s);
+// Around the coarse solves of a call: begin_coarse zeroes their counters, end_coarse waits
+// for the stream and reads them.  The exchange buffers of the grid-wide form are cleared at
+// the first begin and at one that follows a call in which a wait gave up (its CTAs' tags may
+// have run apart) or which left before its end_coarse, on whatever way.
+mg_status begin_coarse(Handle& H, cudaStream_t s);
+mg_status end_coarse(Handle& H, cudaStream_t s, CoopStats* cs);
 template <typename P> mg_status halloc_t(Handle& H, P** p, size_t count) {
     return halloc(H, reinterpret_cast<void**>(p), count * sizeof(P));
 }
