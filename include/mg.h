@@ -83,7 +83,13 @@ typedef struct {
     int parallel;          /* right-hand sides of one mg_solve solved concurrently (1):
                               with > 1, the first right-hand side of a handle builds the
                               deflation space alone, then up to `parallel` solve contexts
-                              (shared hierarchy, own workspaces and streams) share the rest */
+                              (shared hierarchy, own workspaces and streams) share the rest.
+                              Mixed precision with more than 256 coarse sites: the number also
+                              picks the form of the coarsest solve, one grid over the GPU a solve
+                              where the grids of that many solves fit beside one another, else
+                              smaller grids or clusters, whose sums round differently; a handle's
+                              results do not depend on how many of its solves run at a time.
+                              (A server's number is its workers) */
     double partial_tol;    /* 0 (default): V-cycle.  > 0: partial intermediate solve (Section 2
                               variant): the intermediate system is solved to this relative
                               residual (the paper: 0.2) by FGMRES(fgmres_m) preconditioned
@@ -98,8 +104,9 @@ typedef struct {
                               one cluster kernel that streams the coarse operator once for both
                               (mixed precision, V-cycle, deflated coarse solve, device buffers;
                               the paired kernel applies with FP32 FMAs, and the results equal
-                              those of separate solves with coarse_mma = 0).  0 (default): one
-                              right-hand side per worker */
+                              those of separate solves with coarse_mma = 0; where it does not
+                              fit, the two coarsest solves run one after the other as without
+                              pair_rhs).  0 (default): one right-hand side per worker */
     int vcycle_graph;      /* 1 (default): in mixed precision, once the deflation space exists, the
                               V-cycle (grid-0 and grid-1 smoothing and transfers, the coarse
                               GMRES-Proj kernel) is captured into a CUDA graph and replayed: one

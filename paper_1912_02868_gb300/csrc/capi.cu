@@ -352,6 +352,7 @@ mg_status make_context(Handle& P, mg_handle_s** out) {
     C.m0 = P.m0;
     C.p = P.p;
     C.is_context = true;
+    C.peers = P.peers;
     for (int l = 0; l < 3; ++l) {
         C.L64[l] = P.L64[l];
         C.L32[l] = P.L32[l];
@@ -450,6 +451,7 @@ mg_status setup_common(const void* gauge, int Lx, int Lt, double m0, int nvec, i
     H.Lt = Lt;
     H.m0 = m0;
     H.p = p;
+    H.peers = std::max(p.parallel, 1);
     auto fail = [&](mg_status st) {
         free_handle(H);
         delete hs;

@@ -52,6 +52,8 @@ struct CoopArgs {
     long spin;         // try_wait rounds before a dataflow wait gives up (0: the default, 2^20)
     int probe;         // 1 (tests): before the first cycle every CTA waits, bounded by `spin`, on a
                        // barrier that nothing completes, so the give-up path runs (dataflow forms)
+    int peers;         // solves that run beside one another on the GPU, this one among them (coarse
+                       // grids beyond one cluster's 256 sites: picks the launch form)
     int mma;           // 1: the apply runs on tensor cores where it can (coarse_tc.cu: FP32 vectors,
                        // at most 16 sites a CTA, CGS2): FP16 operator times the vector split into
                        // two FP16 parts, FP32 accumulation

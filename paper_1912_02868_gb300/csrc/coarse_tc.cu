@@ -49,7 +49,6 @@ namespace {
 // local memory misses the little L1 that the shared memory leaves).
 constexpr int SD = 2, SD1 = 4;
 constexpr int MAX_SITES = 16;
-constexpr int GRID_SPC = 8;  // grid form: sites a CTA, at least
 constexpr int XW = 48;      // words of one staged site: 12 entry pairs x (hi, hi, lo, lo)
 constexpr int OPA = SD * 3 * 32, OPB = SD1 * 3 * 32;  // fragments of one site in shared memory, by M tile
 
@@ -862,7 +861,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1) k_coarse_tc(const __
 }
 
 struct TcGeometry {
-    int ok = 0, ctas = 0, nw = 0, grid = 0;
+    int ok = 0, ctas = 0, nw = 0, grid = 0, at_once = 1;
     size_t smem = 0;
     TcShape g{};
 };
@@ -948,7 +947,13 @@ void tc_layout(int Nx, int Nt, int ms, int k, int spc, bool two, TcGeometry& G) 
     G.smem = g.ws ? with_w : base;
 }
 
-void tc_geometry_uncached(int Nx, int Nt, int ms, int k, TcGeometry& G) {
+constexpr int GRID_SPC = 8;  // grid form: sites a CTA, at least
+// A step of the grid form, and of coarse_coop.cu's cluster kernel by its sites (18.1 us at
+// 24^2, 29.9 us at 32^2); that kernel's 16-CTA clusters that are resident at once
+constexpr long GRID_STEP_NS = 14000, CLUSTER_STEP_NS = 2900, CLUSTER_SITE_NS = 26;
+constexpr int CLUSTERS = 7;
+
+void tc_geometry_uncached(int Nx, int Nt, int ms, int k, int peers, TcGeometry& G) {
     const int nsite = Nx * Nt;
     if (nsite <= MAX_CLUSTER * MAX_SITES) {
         for (int cl = MAX_CLUSTER; cl >= 1; cl >>= 1) {
@@ -962,22 +967,43 @@ void tc_geometry_uncached(int Nx, int Nt, int ms, int k, TcGeometry& G) {
         }
         return;
     }
-    // grid form: the fewest CTAs that keep a CTA's step short, one per SM
-    G.nw = 16;
-    G.grid = 1;
-    const int most = std::min(sm_count(), GRID_MAX);
-    const int spc = std::max(GRID_SPC, (nsite + most - 1) / most);
-    if (spc > MAX_SITES) return;
-    tc_layout(Nx, Nt, ms, k, spc, false, G);
-    if (G.smem > SMEM_LIMIT) return;
-    int per_sm = 0;
+    // Grid form.  A step takes about as long with eight sites a CTA as with 16 (384^2: 13.3
+    // and 14 us), but a solve then holds twice the SMs, and of solves that run at once only as
+    // many go on as fit: eight sites where all peers' grids fit beside one another, else 16.
+    // Where not even those fit, the cluster kernel (16 CTAs; its step grows with the grid) may
+    // serve the peers sooner: the form with the smaller time a step over the number at once.
+    // Mixed solves, ms each, 8 | 16 sites a CTA | cluster kernel: 7 at once, 320^2 45 | 26 | 25,
+    // 384^2 68 | 39 | 32, 512^2 156 | 79 | 58; 3 at once, 48 | 46 | 50, 69 | 52 | 64,
+    // 152 | 77 | 112; alone, 130 | 127 | 141, 137 | 141 | 179, 157 | 159 | 319.
+    const int sms = sm_count(), most = std::min(sms, GRID_MAX);
+    const int least = (nsite + most - 1) / most;
+    if (least > MAX_SITES) return;
     if (cudaFuncSetAttribute(k_coarse_tc<16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_LIMIT) !=
-            cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_coarse_tc<16, true>, 512, G.smem) != cudaSuccess) {
+        cudaSuccess) {
         (void)cudaGetLastError();
         return;
     }
-    G.ok = per_sm >= 1 && G.ctas <= per_sm * sm_count() ? 1 : 0;
+    for (int spc : {std::max(GRID_SPC, least), MAX_SITES}) {
+        TcGeometry C;
+        C.nw = 16;
+        C.grid = 1;
+        tc_layout(Nx, Nt, ms, k, spc, false, C);
+        if (C.smem > SMEM_LIMIT) continue;
+        int per_sm = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_coarse_tc<16, true>, 512, C.smem) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return;
+        }
+        const int at_once = per_sm * sms / C.ctas;
+        if (at_once < 1) continue;
+        C.ok = 1;
+        C.at_once = at_once;
+        G = C;
+        if (at_once >= peers) return;
+    }
+    if (!G.ok) return;
+    const long grids = std::min(peers, G.at_once), clusters = std::min(peers, CLUSTERS);
+    if (GRID_STEP_NS * clusters > (CLUSTER_STEP_NS + CLUSTER_SITE_NS * nsite) * grids) G.ok = 0;
 }
 
 }  // namespace
@@ -986,11 +1012,13 @@ mg_status launch_coarse_tc(const CoopArgs<float>& a, cudaStream_t s, bool* launc
     *launched = false;
     if (!a.Ah || !a.mma || a.dc || (long)a.Nx * a.Nt > (long)GRID_MAX * MAX_SITES) return MG_OK;
     struct Entry {
-        int dev, Nx, Nt, ms, k;
+        int dev, Nx, Nt, ms, k, peers;
         TcGeometry G;
     };
     static std::mutex mu;
     static std::vector<Entry> cache;
+    // (within one cluster's sites the peers change nothing)
+    const int peers = a.Nx * a.Nt > MAX_CLUSTER * MAX_SITES ? std::min(std::max(a.peers, 1), GRID_MAX) : 1;
     int dev = 0;
     MG_CUDA_TRY(cudaGetDevice(&dev));
     TcGeometry G;
@@ -998,17 +1026,18 @@ mg_status launch_coarse_tc(const CoopArgs<float>& a, cudaStream_t s, bool* launc
         std::lock_guard<std::mutex> lock(mu);
         bool hit = false;
         for (const Entry& e : cache)
-            if (e.dev == dev && e.Nx == a.Nx && e.Nt == a.Nt && e.ms == a.ms && e.k == a.k) {
+            if (e.dev == dev && e.Nx == a.Nx && e.Nt == a.Nt && e.ms == a.ms && e.k == a.k &&
+                e.peers == peers) {
                 G = e.G;
                 hit = true;
                 break;
             }
         if (!hit) {
-            tc_geometry_uncached(a.Nx, a.Nt, a.ms, a.k, G);
-            cache.push_back(Entry{dev, a.Nx, a.Nt, a.ms, a.k, G});
+            tc_geometry_uncached(a.Nx, a.Nt, a.ms, a.k, peers, G);
+            cache.push_back(Entry{dev, a.Nx, a.Nt, a.ms, a.k, peers, G});
         }
     }
-    if (!G.ok || (G.grid && (!a.part || !a.rows))) return MG_OK;
+    if (!G.ok || (G.grid && (!a.part || !a.rows || G.ctas > a.part_ctas))) return MG_OK;
     G.g.part = reinterpret_cast<ulonglong2*>(a.part);
     G.g.rows = reinterpret_cast<ulonglong2*>(a.rows);
     G.g.epoch = a.epoch;

@@ -178,6 +178,7 @@ struct Handle {
     Stats st;
     ApplyTimer timers[3];
     // concurrent solve contexts sharing this hierarchy (mg_solve with nrhs > 1)
+    int peers = 1;                       // solves that run at once beside (and with) this handle's
     bool is_context = false;             // a context: shares hierarchy and deflation, owns workspaces
     cudaStream_t own_stream = nullptr;   // a context's stream
     cudaStream_t work_stream = nullptr;  // this handle's stream for its share of a parallel solve

@@ -354,6 +354,7 @@ void Server::worker_loop() {
             }
             if (st == MG_OK)
                 st = mg_setup(r.gauge, r.L_x, r.L_t, r.m0, pp.nvec, pp.block, &pp, r.starts0, r.starts1, os, &h);
+            if (st == MG_OK) h->h.peers = nworkers;  // workers solve beside one another, on any hierarchy
             if (st == MG_OK) {
                 std::vector<double> bw;
                 const long n0 = (long)r.L_x * r.L_t * 2;

@@ -317,6 +317,7 @@ CoopArgs<T> proj_args(Handle& H, const C2<T>* f, C2<T>* x) {
     a.Ah = std::is_same<T, float>::value ? H.A16c : nullptr;
     a.dc = H.p.coarse_dcgs2;
     a.mma = H.p.coarse_mma;
+    a.peers = H.peers;
     return a;
 }
 
