@@ -239,9 +239,9 @@ __global__ void __launch_bounds__(128) k_stencil_lr_f64_site(double2* __restrict
 
 // FP32 (bound by HBM): one thread per PAIR of dof rows (12 per site), so every
 // operator load is a 16-byte vector of two rows (Q, the self block) or two
-// columns (R).  All of a site's 10.7 KB are on their way at the start: the self block
-// to registers, the hop factors to shared memory by asynchronous copies.  (With the
-// factors loaded where they are used, each block waited for memory three times:
+// columns (R).  STAGED: all of a site's 10.7 KB are on their way at the start, the self
+// block to registers, the hop factors to shared memory by asynchronous copies.  (With the
+// factors loaded where they are used, each block waits for memory three times:
 // 128 x 128 sites, 182 MB, a call with its synchronisation 57.2 -> 51.1 us.)
 // The 16 inner products t = R x_nbr of a site are formed
 // from per-thread partial sums (two entries each) added in shared memory in a
@@ -251,7 +251,16 @@ constexpr int LRF_MAX_SPB = 16;  // sites per block
 constexpr int LRF_HOP4 = 4 * LR_BLOCK / 2;  // 16-byte words of a site's hop factors
 constexpr int LRF_HOPS = LRF_HOP4 + 1;      // their stride in shared memory: sites start on other banks
 size_t lrf_smem(int spb) { return (size_t)spb * LRF_HOPS * sizeof(float4); }
+// Where the factors are staged so.  An operator that stays in L2 from one apply to the next
+// answers a load in less time than the detour through shared memory takes, except on grids
+// of so few sites an SM that one round of loads is the whole apply.  Applies back to back, the
+// best shape of each, staged | loaded where used: 36^2 sites (14 MB) 3.9 | 4.3 us, 44^2 4.7 |
+// 4.7, 64^2 (44 MB) 8.6 | 6.0, 80^2 12.3 | 9.5, 96^2 (99 MB) 19.9 | 19.1, 104^2 (116 MB, L2
+// 129 MB) 26.8 | 30.6, 128^2 36.8 | 41.9.
+constexpr long LRF_FEW_SITES = 12;
+constexpr long LRF_L2_BYTES = 108000000;
 
+template <bool STAGED>
 __global__ void __launch_bounds__(LRF_MAX_SPB* LRF_TPS) k_stencil_lr_f32(float2* __restrict__ y,
                                                                          const float2* __restrict__ x,
                                                                          const float2* __restrict__ F,
@@ -268,14 +277,18 @@ __global__ void __launch_bounds__(LRF_MAX_SPB* LRF_TPS) k_stencil_lr_f32(float2*
     const bool valid = ls < spb && s < nsite;
     const bool flip = dagger && (2 * kt >= N / 2);
     const float4* F4 = reinterpret_cast<const float4*>(F + (valid ? s : 0) * (long)LR_SITE);
-    const float4* hop = lrf_hops + ls * LRF_HOPS;
+    const float4* hop = STAGED ? lrf_hops + ls * LRF_HOPS : F4 + N * N / 2;
+    auto factor = [&](const float4* p) { return STAGED ? *p : __ldg(p); };
     float4 a[N];
     if (valid) {
-        const unsigned dst = (unsigned)__cvta_generic_to_shared(hop);
+        if constexpr (STAGED) {
+            const unsigned dst = (unsigned)__cvta_generic_to_shared(hop);
 #pragma unroll 8
-        for (int q = kt; q < LRF_HOP4; q += LRF_TPS)
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst + 16u * q), "l"(F4 + N * N / 2 + q)
-                         : "memory");
+            for (int q = kt; q < LRF_HOP4; q += LRF_TPS)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst + 16u * q),
+                             "l"(F4 + N * N / 2 + q)
+                             : "memory");
+        }
 #pragma unroll
         for (int l = 0; l < N; ++l) a[l] = __ldg(F4 + l * (N / 2) + kt);  // self block, rows 2 kt, 2 kt + 1
         const int xx = (int)(s % Nx), t = (int)(s / Nx);
@@ -289,7 +302,7 @@ __global__ void __launch_bounds__(LRF_MAX_SPB* LRF_TPS) k_stencil_lr_f32(float2*
             xs[ls][d][kt] = v;
         }
     }
-    asm volatile("cp.async.wait_all;\n" ::: "memory");
+    if constexpr (STAGED) asm volatile("cp.async.wait_all;\n" ::: "memory");
     __syncthreads();
     float2 acc0 = make_float2(0.f, 0.f), acc1 = make_float2(0.f, 0.f);
     if (valid) {
@@ -300,7 +313,7 @@ __global__ void __launch_bounds__(LRF_MAX_SPB* LRF_TPS) k_stencil_lr_f32(float2*
             const float4* R4 = hop + (d * LR_BLOCK + LR_RANK * N) / 2;
 #pragma unroll
             for (int i = 0; i < LR_RANK; ++i) {
-                const float4 r = R4[i * (N / 2) + kt];
+                const float4 r = factor(R4 + i * (N / 2) + kt);
                 float2 p = cfma(make_float2(r.x, r.y), make_float2(xv.x, xv.y), make_float2(0.f, 0.f));
                 p = cfma(make_float2(r.z, r.w), make_float2(xv.z, xv.w), p);
                 part[ls][d * LR_RANK + i][kt] = p;
@@ -333,7 +346,7 @@ __global__ void __launch_bounds__(LRF_MAX_SPB* LRF_TPS) k_stencil_lr_f32(float2*
         const float4* Q4 = hop + d * LR_BLOCK / 2;
 #pragma unroll
         for (int i = 0; i < LR_RANK; ++i) {
-            const float4 q = Q4[i * (N / 2) + kt];
+            const float4 q = factor(Q4 + i * (N / 2) + kt);
             const float2 tv = ts[ls][d * LR_RANK + i];
             acc0 = cfma(make_float2(q.x, q.y), tv, acc0);
             acc1 = cfma(make_float2(q.z, q.w), tv, acc1);
@@ -365,12 +378,17 @@ void launch_stencil_lr(C2<T>* y, const C2<T>* x, const C2<T>* F, const C2<T>* b,
         const long blocks = std::min(sms * waves, nsite);
         const int spb = (shape >= 1 && shape <= LRF_MAX_SPB) ? shape : (int)((nsite + blocks - 1) / blocks);
         const unsigned grid = (unsigned)((nsite + spb - 1) / spb);
+        if (nsite > LRF_FEW_SITES * sms && nsite * (long)(LR_SITE * sizeof(float2)) <= LRF_L2_BYTES) {
+            k_stencil_lr_f32<false><<<grid, spb * LRF_TPS, 0, s>>>(y, x, F, b, Nx, Nt, spb, dagger ? 1 : 0, g);
+            count_launch();
+            return;
+        }
         static std::atomic<bool> set[64];  // shared memory of the largest block allowed, once per device
         int dev = 0;
         if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 && !set[dev].load())
-            set[dev].store(cudaFuncSetAttribute(k_stencil_lr_f32, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            set[dev].store(cudaFuncSetAttribute(k_stencil_lr_f32<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                 (int)lrf_smem(LRF_MAX_SPB)) == cudaSuccess);
-        k_stencil_lr_f32<<<grid, spb * LRF_TPS, lrf_smem(spb), s>>>(y, x, F, b, Nx, Nt, spb, dagger ? 1 : 0, g);
+        k_stencil_lr_f32<true><<<grid, spb * LRF_TPS, lrf_smem(spb), s>>>(y, x, F, b, Nx, Nt, spb, dagger ? 1 : 0, g);
     } else {
         if (nsite < F64_SPLIT_SITES) {
             k_stencil_lr_f64_site<<<(unsigned)nsite, 128, 0, s>>>(y, x, F, b, Nx, Nt, dagger ? 1 : 0, g);
