@@ -43,13 +43,18 @@ constexpr int WILSON_COLS = 2000;
 constexpr int WILSON_SHAPES[] = {64, 128, 256, WILSON_TILE + 4, WILSON_TILE + 8, WILSON_COLS + 2, WILSON_COLS + 4};
 constexpr int STENCIL_F32_SHAPES[] = {4, 8, 16, 24, 32};
 constexpr int STENCIL_LR_F32_SHAPES[] = {4, 8, 12, 16};
-// FP64 stencils of fewer sites than this take one CTA a site, its columns split over the
-// warps.  An FP64 instruction of a warp holds its scheduler for 64 cycles, so a site's
-// time is its instructions on the busiest scheduler: a quarter of them when four warps
-// share it.  With a CTA's worth of sites for every SM the eight-site blocks use as many
-// schedulers and need fewer instructions.  Measured: the dense stencil on 20 x 12 sites
-// 24.8 us in eight-site blocks, 7.7 us so; the factored one on 16 x 16 sites 6.5 us.
-constexpr long F64_SPLIT_SITES = 2048;
+// Whether an FP64 stencil takes one CTA a site, its columns split over four warps, or blocks
+// of eight sites.  An FP64 instruction of a warp holds its scheduler for 64 cycles, so a
+// site's time is its instructions on the busiest scheduler: a quarter of them when four warps
+// share it.  Split, the time grows with the sites of an SM (q); a wave of blocks, eight sites
+// on every SM, takes as long full as nearly empty.  The split form to q = per_wave * waves +
+// extra, within two waves.  Measured, split | blocks: the dense stencil (7, 0) 24.6 | 26.2 us at
+// q = 7, 27.5 | 26.2 at 8, 34.0 | 48.6 at 10, 47.5 | 50.3 at 14; the factored one (5, 1) 15.0 |
+// 15.4 at q = 6, 17.4 | 15.4 at 7, 23.8 | 27.3 at 10, 32.4 | 27.4 at 14.
+inline bool f64_split_sites(long nsite, int per_wave, int extra) {
+    const long sms = sm_count(), q = (nsite + sms - 1) / sms, waves = (q + 7) / 8;
+    return waves <= 2 && q <= per_wave * waves + extra;
+}
 
 // ---------------------------------------------------------------- wilson ----
 // y = D x, D^+ x (dagger), or y = b - D x when b != nullptr.  Section 2.

@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(SPB* N) k_stencil(C2<T>* __restrict__ y, const
     y[s * N + k] = acc;
 }
 
-// FP64, one CTA a site (F64_SPLIT_SITES): thread (d, k) sums direction d of row k, then
+// FP64, one CTA a site (f64_split_sites): thread (d, k) sums direction d of row k, then
 // the five directions are added in order, each real component on its own thread.  Bound
 // by the FP64 pipe (four warps of 24 complex FMAs, 6.1k cycles at 64 a warp
 // instruction): 7.7 us an apply on 20 x 12 sites, 24.8 us with eight sites a block.
@@ -182,7 +182,7 @@ void launch_stencil(C2<T>* y, const C2<T>* x, const C2<T>* A, const C2<T>* b, in
         const unsigned grid = (unsigned)((nsite + spb - 1) / spb);
         k_stencil_f32<<<grid, spb * F32_TPS, 0, s>>>(y, x, A, b, Nx, Nt, spb, dagger ? 1 : 0, g);
     } else {
-        if (nsite < F64_SPLIT_SITES) {
+        if (f64_split_sites(nsite, 7, 0)) {
             k_stencil_f64_site<<<(unsigned)nsite, 128, 0, s>>>(y, x, A, b, Nx, Nt, dagger ? 1 : 0, g);
             count_launch();
             return;

@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(LR_SPB* N) k_stencil_lr(C2<T>* __restrict__ y,
 }
 
 
-// FP64, one CTA of four warps a site (F64_SPLIT_SITES): warp d forms t = R x_nbr of hop
+// FP64, one CTA of four warps a site (f64_split_sites): warp d forms t = R x_nbr of hop
 // direction d + 1 (lane (i, p) three columns of rank i, eight lanes a product), adds
 // Q t to its quarter of the self block's columns, and the four warps' sums are added in
 // order, each real component on its own thread.  Bound by the FP64 pipe and three
@@ -390,7 +390,7 @@ void launch_stencil_lr(C2<T>* y, const C2<T>* x, const C2<T>* F, const C2<T>* b,
                                                 (int)lrf_smem(LRF_MAX_SPB)) == cudaSuccess);
         k_stencil_lr_f32<true><<<grid, spb * LRF_TPS, lrf_smem(spb), s>>>(y, x, F, b, Nx, Nt, spb, dagger ? 1 : 0, g);
     } else {
-        if (nsite < F64_SPLIT_SITES) {
+        if (f64_split_sites(nsite, 5, 1)) {
             k_stencil_lr_f64_site<<<(unsigned)nsite, 128, 0, s>>>(y, x, F, b, Nx, Nt, dagger ? 1 : 0, g);
             count_launch();
             return;

@@ -1,7 +1,8 @@
-"""The intermediate stencil at the sizes where its FP32 kernel changes: hop factors staged in
+"""The intermediate stencil at the sizes where its kernels change: FP32 hop factors staged in
 shared memory (few sites an SM, or an operator larger than L2) or loaded where they are used,
-and the dense blocks beside it.  Against the dense blocks of mg_get_stencil in FP64, max norm
-2e-6 (FP32) and 1e-12 (FP64), the bounds of the operator applies; D and D^+.
+FP64 one CTA a site or blocks of eight, factored and dense.  Against the dense blocks of
+mg_get_stencil in FP64, max norm 2e-6 (FP32) and 1e-12 (FP64), the bounds of the operator
+applies; D and D^+.
 """
 import pytest
 
@@ -24,9 +25,11 @@ def _apply(A, x, dagger):
     return y * sign
 
 
-# sites (a GB300 has 152 SMs): 16, 1728 and 1920 (staged to 12 an SM, 1824), 10000 and 10400
-# (107.5 and 111.8 MB of factors)
-@pytest.mark.parametrize("nx,nt", [(4, 4), (36, 48), (40, 48), (100, 100), (104, 100)])
+# sites (a GB300 has 152 SMs): 16, 1728 and 1920 (FP32: staged to 12 an SM, 1824), 10000 and 10400
+# (107.5 and 111.8 MB of FP32 factors); FP64, sites an SM: 864 (6), 1024 (7), 1152 (8), 1600 (11),
+# 1760 (12), 2112 (14), 2304 (16)
+@pytest.mark.parametrize("nx,nt", [(4, 4), (36, 48), (40, 48), (100, 100), (104, 100), (36, 24), (32, 32), (32, 36),
+                                   (40, 40), (40, 44), (44, 48), (48, 48)])
 def test_kernel_boundaries(cuda_lib, nx, nt):
     import torch
     import paper_1912_02868_gb300 as mg
