@@ -322,8 +322,10 @@ __device__ unsigned tc_clock_launches = 0;
 #endif
 
 // NW warps.  NW = 8 serves at most 8 sites a CTA at two CTAs per SM, NW = 16 at most
-// 16 (128 registers a thread either way).
-template <int NW, bool GRID>
+// 16 (128 registers a thread either way).  PROBE: the test probe's wait comes first.  It is
+// an instantiation of its own because its code, though never run, changed the others': a
+// 384^2 solve 135.8 instead of 133.5 ms, 512^2 158.7 instead of 155.0, 256^2 51.9 instead of 51.8.
+template <int NW, bool GRID, bool PROBE>
 __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1) k_coarse_tc(const __grid_constant__ CoopArgs<float> a,
                                                                         const __grid_constant__ TcShape g) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -466,7 +468,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1) k_coarse_tc(const __
         V[tid] = a.f[(long)s0 * NDOF + tid];
     }
     __syncthreads();
-    if (a.probe) {  // test probe: a wait that nothing ends gives up
+    if constexpr (PROBE) {  // test probe: a wait that nothing ends gives up
         const long spin = a.spin > 0 ? a.spin : FLOW_SPIN;
         if constexpr (GRID) {
             if (tid == 0) {
@@ -766,19 +768,22 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1) k_coarse_tc(const __
             }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) h2n += __shfl_xor_sync(0xffffffffu, h2n, o);
-            const float hn = sqrtf(fmaxf(S.nrm[1] - h2n, 0.f)), inv = hn > 0.f ? 1.f / hn : 0.f;
+            const float hh = fmaxf(S.nrm[1] - h2n, 0.f);
             TC_STAMP(10);
             arm(2, S.nremote * XW * 4);
             if (warp * 32 < nrows) {
                 float2 v = make_float2(0.f, 0.f);
                 if (row_on) {
+                    // the rows need the reciprocal root and the least squares (a warp without rows)
+                    // the root: each forms its own
+                    const float inv = hh > 0.f ? __frsqrt_rn(hh) : 0.f;
                     v = cscale(csub(wl[tid], tc_combine<false>(V + tid, ldv, S.red[1], j + 1)), inv);
                     wl[tid] = v;
                 }
                 TC_STAMP(11);
                 stage(v);
             }
-            if (warp == NW - 1) ls_update(j, hn);
+            if (warp == NW - 1) ls_update(j, sqrtf(hh));
             TC_STAMP(5);
 #ifdef CP_PHASE_CLOCKS
             ++clk_steps;
@@ -886,16 +891,21 @@ int max_halo(int Nx, int Nt, int spc) {
     return most;
 }
 
+// the shared memory and, of the cluster form, the cluster size that a kernel may have
+template <int NW, bool GRID, bool PROBE>
+bool allow() {
+    auto* kern = k_coarse_tc<NW, GRID, PROBE>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_LIMIT) == cudaSuccess &&
+        (GRID || cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess))
+        return true;
+    (void)cudaGetLastError();
+    return false;
+}
+
 template <int NW>
 bool fits(TcGeometry& G) {
-    auto* kern = k_coarse_tc<NW, false>;
-    {
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_LIMIT) != cudaSuccess ||
-            cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-            (void)cudaGetLastError();
-            return false;
-        }
-    }
+    auto* kern = k_coarse_tc<NW, false, false>;
+    if (!allow<NW, false, false>()) return false;
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -978,11 +988,7 @@ void tc_geometry_uncached(int Nx, int Nt, int ms, int k, int peers, TcGeometry& 
     const int sms = sm_count(), most = std::min(sms, GRID_MAX);
     const int least = (nsite + most - 1) / most;
     if (least > MAX_SITES) return;
-    if (cudaFuncSetAttribute(k_coarse_tc<16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_LIMIT) !=
-        cudaSuccess) {
-        (void)cudaGetLastError();
-        return;
-    }
+    if (!allow<16, true, false>()) return;
     for (int spc : {std::max(GRID_SPC, least), MAX_SITES}) {
         TcGeometry C;
         C.nw = 16;
@@ -990,7 +996,8 @@ void tc_geometry_uncached(int Nx, int Nt, int ms, int k, int peers, TcGeometry& 
         tc_layout(Nx, Nt, ms, k, spc, false, C);
         if (C.smem > SMEM_LIMIT) continue;
         int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_coarse_tc<16, true>, 512, C.smem) != cudaSuccess) {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_coarse_tc<16, true, false>, 512, C.smem) !=
+            cudaSuccess) {
             (void)cudaGetLastError();
             return;
         }
@@ -1057,9 +1064,19 @@ mg_status launch_coarse_tc(const CoopArgs<float>& a, cudaStream_t s, bool* launc
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (G.grid) MG_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_coarse_tc<16, true>, a, G.g));
-    else if (G.nw == 8) MG_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_coarse_tc<8, false>, a, G.g));
-    else MG_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_coarse_tc<16, false>, a, G.g));
+    if (a.probe) {
+        const bool ok = G.grid ? allow<16, true, true>() : G.nw == 8 ? allow<8, false, true>() : allow<16, false, true>();
+        if (!ok) return set_error("coarse solve: the probed kernel cannot run here"), MG_ECUDA;
+        if (G.grid) MG_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_coarse_tc<16, true, true>, a, G.g));
+        else if (G.nw == 8) MG_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_coarse_tc<8, false, true>, a, G.g));
+        else MG_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_coarse_tc<16, false, true>, a, G.g));
+    } else if (G.grid) {
+        MG_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_coarse_tc<16, true, false>, a, G.g));
+    } else if (G.nw == 8) {
+        MG_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_coarse_tc<8, false, false>, a, G.g));
+    } else {
+        MG_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_coarse_tc<16, false, false>, a, G.g));
+    }
     count_launch();
     *launched = true;
     return MG_OK;
