@@ -1127,7 +1127,7 @@ def run_micro(args):
                     if i:
                         ms.append(time.perf_counter() - t0)
                 t = float(np.mean(ms))
-                out = {"kernel": "k_cb_cycle", "coarse_sites": (Lm // 16) ** 2, "nrhs": nb, "ms": t * 1e3,
+                out = {"kernel": "batched coarse cycle", "coarse_sites": (Lm // 16) ** 2, "nrhs": nb, "ms": t * 1e3,
                        "steps": int(max(it)), "us_per_step": t * 1e6 / max(it)}
             print(json.dumps(out), flush=True)
     finally:

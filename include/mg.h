@@ -297,12 +297,14 @@ enum { MG_COARSE_PROBE_TIMEOUT = 1 };
 
 /* launch shape of the last mg_coarse_solve */
 typedef struct {
-    int ctas;            /* CTAs of the cluster */
+    int ctas;            /* CTAs of the cluster, or of the grid (more than 256 coarse sites) */
     int sites_per_cta;   /* coarse sites each CTA owns */
-    int dataflow;        /* 1: st.async / byte-counted mbarrier exchange in each Arnoldi step */
+    int dataflow;        /* 1: each Arnoldi step's values are awaited themselves, without barriers:
+                            st.async and byte-counted mbarriers in a cluster, tagged words in a grid */
     int dcgs2;           /* 1: delayed CGS2 ran (one exchange per step) */
     int half_operator;   /* 1: the FP16 copy of the operator was streamed */
-    int shared_blocks;   /* 1: the FP16 blocks of three directions were held in shared memory */
+    int shared_blocks;   /* 1: FP16 blocks were held on chip (three directions in shared memory; with
+                            tensor_apply all five, in shared memory and registers) */
     int paired;          /* 1: the two-right-hand-side kernel */
     long long cycles;    /* GMRES cycles of right-hand side 0 */
     long long timeouts;  /* CTAs in which a bounded wait gave up */
@@ -323,9 +325,9 @@ typedef struct {
  *              with MG_BF16 / MG_F16
  *   b, x       device, [nrhs][n_2] in that precision; x is output
  *   flags      MG_COARSE_PROBE_TIMEOUT (tests): before the first cycle every CTA
- *              waits, bounded by `spin`, on a barrier that nothing completes, so
- *              the give-up path runs; the call then returns MG_ETIMEOUT and the
- *              handle stays usable.  MG_BF16 / MG_F16: every CTA of the batched
+ *              waits, bounded by `spin`, on a barrier that nothing completes (a
+ *              word that nothing writes, in a grid), so the give-up path runs; the
+ *              call then returns MG_ETIMEOUT and the handle stays usable.  MG_BF16 / MG_F16: every CTA of the batched
  *              cycle kernel waits so at the start of each cycle (info->timeouts
  *              = 1); the probe needs the cycle kernel's resident grid (MG_EINVAL
  *              on coarse grids that run the three-kernel steps)

@@ -14,10 +14,14 @@
 // The arithmetic is that of the kernels it replaces: sums in the vectors' precision,
 // the norm from its own pass after the second update, the least squares in FP64.
 //
-// Sizes: FP32 up to 131072 entries (the fine grid of 256^2), 16 a thread: there k_arnoldi
-// takes 20.1 us, the kernels it replaces 25.7 us and five gaps.  Longer vectors would
-// spill w, and 16 SMs then bound them.  FP64 up to 16384, two a thread, because the FP64
-// pipe of 16 SMs bounds longer ones: at 8192 entries 29.9 us against 26.7 us and the gaps.
+// Sizes: FP32 up to 131072 entries (the fine grid of 256^2), 16 a thread.  Steps in a
+// captured graph, this kernel | those it replaces: 24576 entries 14.7 | 21.3 us, 65536 15.9 |
+// 21.7, 131072 20.9 | 25.6 (the first two steps; over eight 29.3 | 32.1).  Longer vectors
+// would spill w, and 16 SMs then bound them.  FP64 up to 16384, two a thread.  There the FP64
+// pipe of 16 SMs bounds it: 4096 entries 22.2 | 24.8 us, 8192 31.4 | 25.0, 16384 41.7 | 26.8.
+// But FP64 steps are launched one by one, and the host takes as long for six launches as the
+// longer kernel does: FP64 solves with the limit at 16384 | 8192 | 5120 entries, 64^2 74.7 |
+// 74.6 | 76.7 ms, 80 x 64 101.7 | 102.1 | 103.0, 128 x 64 131.5 | 131.5 | 131.5.
 // A 256^2 mixed solve 58.8 -> 56.1 ms, a 128^2 partial solve 25.2 -> 21.1 ms, a 64^2 FP64
 // solve 83.9 -> 80.4 ms.
 #include <cooperative_groups.h>
