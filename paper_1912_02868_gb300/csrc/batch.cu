@@ -24,6 +24,9 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <atomic>
+#include <type_traits>
+
 #include "batch.cuh"
 
 namespace mg {
@@ -423,11 +426,13 @@ __global__ void k_pack_frag(unsigned* out, const double2* __restrict__ A, long n
 // sides).  The operator of a group's sites (11.5 KB a site) is staged in shared memory
 // once (cp.async), so every tile of a site reads the same copy; each warp issues all
 // its neighbour-vector loads before it waits.  A CTA takes groups blockIdx.x, + gridDim.x,
-// ... and stages the next one while it multiplies (two buffers, unless every CTA has one
-// group only): without it nothing was in flight during the products.  That and the
+// ... and stages the next one while it multiplies (WALK, two buffers): without it nothing
+// was in flight during the products.  That and the
 // fragment order (a third of the instructions that formed both rows of a word):
-// 128 x 128 sites x 16 right-hand sides, FP16, 289 MB: 77.8 -> 68.9 us.
-template <bool F16, bool RES>
+// 128 x 128 sites x 16 right-hand sides, FP16, 289 MB: 77.8 -> 68.9 us.  Where every CTA has
+// one group only the kernel has no loop and no registers for it (102 instead of 127): 8
+// right-hand sides on those sites 49.9 -> 48.7 us.
+template <bool F16, bool RES, bool WALK>
 __global__ void __launch_bounds__(256, 2) k_bstencil_mma(float2* __restrict__ Y, const float2* __restrict__ X,
                                                          const float2* __restrict__ B, long vr,
                                                          const unsigned* __restrict__ Af, int Nx, int Nt, int ntiles,
@@ -469,9 +474,13 @@ __global__ void __launch_bounds__(256, 2) k_bstencil_mma(float2* __restrict__ Y,
                 }
             }
         }
-        if (grp + (int)gridDim.x < ngroups) stage(grp + gridDim.x, buf ^ 1);
-        asm volatile("cp.async.commit_group;\n" ::: "memory");
-        asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+        if constexpr (WALK) {
+            if (grp + (int)gridDim.x < ngroups) stage(grp + gridDim.x, buf ^ 1);
+            asm volatile("cp.async.commit_group;\n" ::: "memory");
+            asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+        }
         __syncthreads();
         if (run) {
             float acc[3][4];
@@ -514,6 +523,7 @@ __global__ void __launch_bounds__(256, 2) k_bstencil_mma(float2* __restrict__ Y,
                 }
             }
         }
+        if constexpr (!WALK) break;  // one group a CTA
         __syncthreads();  // the buffer is free for the group after the next
     }
 }
@@ -591,23 +601,22 @@ void launch_bstencil_mma(float2* Y, const float2* X, const float2* B, long vr, c
     const bool walk = G <= 4 && groups > 2L * sm_count();
     const unsigned grid = (unsigned)(walk ? 2L * sm_count() : groups);
     const size_t smem = (size_t)(walk ? 2 : 1) * G * SITE_WORDS * sizeof(unsigned);
-    static bool attr_set[64] = {};  // larger than the default 48 KB when G > 4
+    auto pick = [&](auto f16, auto res) {
+        constexpr bool F = decltype(f16)::value, R = decltype(res)::value;
+        return walk ? &k_bstencil_mma<F, R, true> : &k_bstencil_mma<F, R, false>;
+    };
+    const std::true_type yes{};
+    const std::false_type no{};
+    auto* kern = fp16 ? (B ? pick(yes, yes) : pick(yes, no)) : (B ? pick(no, yes) : pick(no, no));
+    // larger than the default 48 KB when G > 4 or with two buffers
+    const int mx = 8 * SITE_WORDS * (int)sizeof(unsigned);
+    static std::atomic<bool> attr_set[64][8];  // once per device and kernel
+    const int which = (fp16 ? 4 : 0) + (B ? 2 : 0) + (walk ? 1 : 0);
     int dev = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 && !attr_set[dev]) {
-        const int mx = 8 * SITE_WORDS * (int)sizeof(unsigned);
-        cudaFuncSetAttribute(k_bstencil_mma<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-        cudaFuncSetAttribute(k_bstencil_mma<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-        cudaFuncSetAttribute(k_bstencil_mma<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-        cudaFuncSetAttribute(k_bstencil_mma<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-        attr_set[dev] = true;
-    }
-    if (fp16) {
-        if (B) k_bstencil_mma<true, true><<<grid, 256, smem, s>>>(Y, X, B, vr, Af, Nx, Nt, ntiles, g);
-        else k_bstencil_mma<true, false><<<grid, 256, smem, s>>>(Y, X, B, vr, Af, Nx, Nt, ntiles, g);
-    } else {
-        if (B) k_bstencil_mma<false, true><<<grid, 256, smem, s>>>(Y, X, B, vr, Af, Nx, Nt, ntiles, g);
-        else k_bstencil_mma<false, false><<<grid, 256, smem, s>>>(Y, X, B, vr, Af, Nx, Nt, ntiles, g);
-    }
+    if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 && !attr_set[dev][which].load())
+        attr_set[dev][which].store(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, mx) ==
+                                   cudaSuccess);
+    kern<<<grid, 256, smem, s>>>(Y, X, B, vr, Af, Nx, Nt, ntiles, g);
     count_launch();
 }
 
